@@ -196,14 +196,23 @@ __global__ void phi4_init_kernel(F4* phi, int64_t n, sw::KeySchedule ks, int col
   }
 }
 
+__device__ __forceinline__ uint32_t abs_high(double d) { return (uint32_t)__double2hiint(d) & 0x7fffffffu; }
+
 // The projections in binary64 and, for the bond kernel's first test, rounded
 // to binary32.
-__global__ void phi4_project_kernel(const F4* phi, double* a, float* af, int* par, int64_t n, Dir d) {
+__global__ void phi4_project_kernel(const F4* phi, double* a, float* af, int* par, int64_t n, Dir d, uint32_t* top) {
+  uint32_t big = 0u;  // high word of the largest |component|
   GRID_LOOP(x, n) {
-    const double v = proj(phi[x], d);
+    const F4 f = phi[x];
+    const double v = proj(f, d);
     a[x] = v;
     af[x] = __double2float_rn(v);
     par[x] = (int)x;
+    big = max(max(max(big, abs_high(f.x)), abs_high(f.y)), max(abs_high(f.z), abs_high(f.w)));
+  }
+  if (top) {
+    big = __reduce_max_sync(0xffffffffu, big);
+    if ((threadIdx.x & 31) == 0) atomicMax(top, big);
   }
 }
 
@@ -272,9 +281,71 @@ __global__ void phi4_reflect_kernel(F4* phi, const double* a, const int* par, co
   }
 }
 
-__global__ void phi4_observe_kernel(const F4* phi, int L, int64_t n, double* out /* E, M0..M3 */) {
-  double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  GRID_LOOP(i, n) {
+// ------------------------------------------------------------ E and M
+//
+// E and M of the new field. GB300's binary64 rate is about 1/60 of its
+// integer rate, and E takes 24 binary64 operations a site: at L = 64 the
+// binary64 kernel below ran 739 us, all of it in that pipe; the fixed-point one
+// runs 223 us (16.8M sites, 0.54 GB of field), bound by instruction issue.
+// Large lattices therefore sum in 64-bit fixed point: with 2^T above every |phi| (T from the
+// largest component, which the projection kernel leaves in *top; a reflection
+// keeps the length of phi), a component c becomes the integer nearest to
+// c 2^(54-T) -- exact for components down to 2^-2 of the bound, else rounded by
+// at most 2^-55 of it -- and from there on everything is exact: neighbour sums
+// and M are integer sums, and phi . S (S the sum of the four forward
+// neighbours) is taken from 27-bit low and signed high parts, each of the
+// partial products in a 64-bit sum of its own. |phi| < 2^54 and |S| < 2^56 in
+// these units, so by Cauchy-Schwarz a site adds less than 2^56 to the high
+// products, 2^58 to the mixed and 2^56 to the low ones, and sixteen sites fit.
+
+struct Fix4 {
+  int64_t v[4];
+};
+
+// d 2^(54-T) rounded to an integer; shift0 = T + 1031. A double is m 2^(e - 1086)
+// with m its mantissa from bit 63 down, so the result is m >> (T + 1032 - e),
+// taken with one more bit, given its sign and rounded.
+__device__ __forceinline__ int64_t to_fixed(double d, int shift0) {
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  const uint64_t m = ((uint64_t)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
+  const uint32_t sh = (uint32_t)(shift0 - (int)((hi >> 20) & 0x7ffu));
+  uint64_t x;
+  asm("shr.b64 %0, %1, %2;" : "=l"(x) : "l"(m), "r"(sh));  // shifts past 63 give 0
+  const int s = (int32_t)hi >> 31;
+  return (((int64_t)x ^ s) + (1 - s)) >> 1;
+}
+__device__ __forceinline__ Fix4 to_fixed(const F4& f, int shift0) {
+  return Fix4{{to_fixed(f.x, shift0), to_fixed(f.y, shift0), to_fixed(f.z, shift0), to_fixed(f.w, shift0)}};
+}
+
+// Adds the block's sums of v[0..4] to out[0..4]. The five values are reduced
+// together: two of them share each of the first three exchange steps (a lane
+// keeps one and passes the other on), so a warp takes 8 binary64 additions
+// instead of 25 (this pipe bounds the kernels that end here).
+__device__ __forceinline__ void block_add5(const double v[5], double* out) {
+  __shared__ double red[5][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto pass = [&](double keep0, double keep1, int bit) {  // lanes with the bit keep the second value
+    const bool up = (lane & bit) != 0;
+    return (up ? keep1 : keep0) + __shfl_xor_sync(0xffffffffu, up ? keep0 : keep1, bit);
+  };
+  const double p = pass(v[0], v[1], 1), q = pass(v[2], v[3], 1), r = v[4] + __shfl_xor_sync(0xffffffffu, v[4], 1);
+  const double pq = pass(p, q, 2), rr = r + __shfl_xor_sync(0xffffffffu, r, 2);
+  double w = pass(pq, rr, 4);  // lane bits 2..0: 000 v0, 001 v1, 010 v2, 011 v3, 1xx v4
+  w += __shfl_xor_sync(0xffffffffu, w, 8);
+  w += __shfl_xor_sync(0xffffffffu, w, 16);
+  if (lane < 5) red[lane][warp] = w;
+  __syncthreads();
+  if (threadIdx.x < 5) {
+    double s = 0.0;
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += red[threadIdx.x][k];
+    atomicAdd(out + threadIdx.x, s);
+  }
+}
+
+// Binary64 sums of the sites x0, x0 + step, ... below n.
+__device__ void observe_binary64(const F4* phi, int L, int64_t n, int64_t x0, int64_t step, double v[5]) {
+  for (int64_t i = x0; i < n; i += step) {
     const uint32_t x = (uint32_t)i;
     const Coords k = coords_of(x, (uint32_t)L);
     const F4 f = phi[x];
@@ -289,21 +360,94 @@ __global__ void phi4_observe_kernel(const F4* phi, int L, int64_t n, double* out
     v[3] += f.z;
     v[4] += f.w;
   }
-  __shared__ double red[5][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    double s = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[k][warp] = s;
+}
+
+__global__ void phi4_observe_kernel(const F4* phi, int L, int64_t n, double* out /* E, M0..M3 */) {
+  double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  observe_binary64(phi, L, n, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, v);
+  block_add5(v, out);
+}
+
+// A block takes kObserveThreads consecutive sites of the (x0, x1, x2) volume
+// and marches `steps` slices up x3: a thread's next slice is the x3 neighbour
+// of its current one, and the x0 and x1 neighbours are mostly other threads'
+// sites, passed as integers in shared memory (two slices' buffers, so one
+// barrier a slice). Only the x2 neighbour, and those past the block's range,
+// are loaded and converted again: 2.25 conversions a site at L = 64.
+constexpr int kObserveThreads = 256;
+constexpr int kObserveSteps = 16;
+// From 2^20 sites: below, the binary64 kernel takes 10 us or less (L = 16), most
+// of it latency, and the fixed-point one has too few blocks of sixteen slices.
+constexpr int64_t kObserveFixedSites = 1 << 20;
+
+__global__ void __launch_bounds__(kObserveThreads)
+    phi4_observe_fixed_kernel(const F4* phi, int L, int64_t n, const uint32_t* top, int steps, double* out) {
+  const int et = (int)(*top >> 20);  // biased exponent of the largest component before the reflection
+  if (et < 1023 - 400 || et > 1023 + 400) {
+    // zero, subnormal, huge, infinite or NaN components: the binary64 sums
+    double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    const int64_t b = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
+    observe_binary64(phi, L, n, b * blockDim.x + threadIdx.x, (int64_t)gridDim.x * gridDim.y * blockDim.x, v);
+    block_add5(v, out);
+    return;
   }
-  __syncthreads();
-  if (threadIdx.x < 5) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[threadIdx.x][w];
-    atomicAdd(out + threadIdx.x, s);
+  const int T = et - 1023 + 2;        // |phi| <= 2 max component < 2^T
+  const int shift0 = T + 1031;
+  __shared__ longlong2 s_x[2][2][kObserveThreads];
+  const uint32_t V = (uint32_t)L * L * L, s0 = blockIdx.x * kObserveThreads, s = s0 + threadIdx.x;
+  const bool have = s < V;
+  const uint32_t sc = have ? s : V - 1;
+  const Coords k = coords_of(sc, (uint32_t)L);
+  const uint32_t n0 = nb(sc, 0, k, L, 1), n1 = nb(sc, 1, k, L, L), n2 = sc + (k.c[2] + 1 == (uint32_t)L ? L * L - V : L * L);
+  const bool in0 = n0 - s0 < kObserveThreads, in1 = n1 - s0 < kObserveThreads;
+  const int z0 = blockIdx.y * steps, z1 = min(z0 + steps, L);
+  int64_t hh = 0, cr = 0, ll = 0, m[4] = {0, 0, 0, 0};
+  Fix4 own = to_fixed(phi[(size_t)z0 * V + sc], shift0);
+  for (int z = z0; z < z1; ++z) {
+    const F4* slice = phi + (size_t)z * V;
+    const Fix4 up = to_fixed(phi[(size_t)(z + 1 == L ? 0 : z + 1) * V + sc], shift0);
+    const F4 g2 = slice[n2];
+    longlong2(&buf)[2][kObserveThreads] = s_x[z & 1];
+    buf[0][threadIdx.x] = make_longlong2(own.v[0], own.v[1]);
+    buf[1][threadIdx.x] = make_longlong2(own.v[2], own.v[3]);
+    Fix4 S = to_fixed(g2, shift0);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) S.v[c] += up.v[c];
+    __syncthreads();
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      const uint32_t nbr = d ? n1 : n0;
+      Fix4 g;
+      if (d ? in1 : in0) {
+        const longlong2 u = buf[0][nbr - s0], w = buf[1][nbr - s0];
+        g = Fix4{{u.x, u.y, w.x, w.y}};
+      } else {
+        g = to_fixed(slice[nbr], shift0);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) S.v[c] += g.v[c];
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int xh = (int)(own.v[c] >> 27), Sh = (int)(S.v[c] >> 27);
+      const int xl = (int)own.v[c] & 0x7ffffff, Sl = (int)S.v[c] & 0x7ffffff;
+      hh += (int64_t)xh * Sh;
+      cr += (int64_t)xh * Sl + (int64_t)xl * Sh;
+      ll += (int64_t)xl * Sl;
+      m[c] += own.v[c];
+    }
+    own = up;
   }
+  double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  if (have) {
+    // E = hh 2^54 + cr 2^27 + ll, rounded to a multiple of 2^54 (2^-54 of a site's bound)
+    hh += (cr + ((ll + (1 << 26)) >> 27) + (1 << 26)) >> 27;
+    v[0] = (double)hh * scalbn(1.0, 2 * T - 54);
+    const double u = scalbn(1.0, T - 54);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[1 + c] = (double)m[c] * u;
+  }
+  block_add5(v, out);
 }
 
 int grid_of(int64_t n) {
@@ -336,6 +480,7 @@ struct sw_phi4 {
   uint8_t* bonds = nullptr;
   uint8_t* flip = nullptr;
   double* obs = nullptr;  // [cap][5]: E, M0..M3
+  uint32_t* top = nullptr;  // high word of the field's largest |component| (projection -> E and M)
   int* err = nullptr;
 };
 
@@ -351,7 +496,7 @@ namespace {
   } while (0)
 
 void free_phi4(sw_phi4* h) {
-  void* ptrs[] = {h->phi, h->a, h->af, h->par, h->bonds, h->flip, h->obs, h->err};
+  void* ptrs[] = {h->phi, h->a, h->af, h->par, h->bonds, h->flip, h->obs, h->top, h->err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -408,7 +553,9 @@ int direction(uint64_t seed, uint32_t t, double r[4]) {
 int clusters(sw_phi4* h, Dir& d) {
   if (direction(h->seed, (uint32_t)h->t, d.r) != 0) return ffail(SW_EDEVICE, "no direction found");
   const int g = grid_of(h->n);
-  phi4_project_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->af, h->par, h->n, d);
+  uint32_t* const top = h->n >= kObserveFixedSites ? h->top : nullptr;
+  if (top) F_CUDA(cudaMemsetAsync(top, 0, sizeof(uint32_t), h->stream), "range word");
+  phi4_project_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->af, h->par, h->n, d, top);
   phi4_bonds_kernel<<<g, 256, 0, h->stream>>>(h->a, h->af, h->bonds, h->L, h->n, 4.0 * h->kappa, (uint32_t)h->t,
                                               h->ks);
   phi4_unite_kernel<<<g, 256, 0, h->stream>>>(h->bonds, h->par, h->L, h->n, h->err);
@@ -459,6 +606,7 @@ int sw_phi4_create(int32_t L, double kappa, uint64_t seed, int32_t init, void* s
   if (e == cudaSuccess) e = cudaMalloc(&h->par, n * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->bonds, n);
   if (e == cudaSuccess) e = cudaMalloc(&h->flip, n);
+  if (e == cudaSuccess) e = cudaMalloc(&h->top, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&h->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int), h->stream);
   if (e == cudaSuccess) {
@@ -494,7 +642,13 @@ int sw_phi4_sweep(sw_phi4* h, int32_t n) {
     double* o = h->obs + 5 * (h->t - h->t_base);
     F_CUDA(cudaMemsetAsync(o, 0, 5 * sizeof(double), h->stream), "trace row");
     phi4_reflect_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->par, h->flip, h->n, d);
-    phi4_observe_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->L, h->n, o);
+    if (h->n >= kObserveFixedSites) {
+      const int V = h->L * h->L * h->L;
+      const dim3 grid((V + kObserveThreads - 1) / kObserveThreads, (h->L + kObserveSteps - 1) / kObserveSteps);
+      phi4_observe_fixed_kernel<<<grid, kObserveThreads, 0, h->stream>>>(h->phi, h->L, h->n, h->top, kObserveSteps, o);
+    } else {
+      phi4_observe_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->L, h->n, o);
+    }
     F_CUDA(cudaGetLastError(), "phi4 reflect launch");
     h->t += 1;
   }
