@@ -5,24 +5,24 @@
 // One update at counter t:
 //   host      the direction r, uniform on the 3-sphere (O3), by rejection
 //             from Philox blocks, computed on the host;
-//   project   a thread per site: a_x = phi_x . r; every site starts as its
-//             own root;
-//   bonds     a thread per site draws the words of block (x, t, 4, 0) and
-//             bonds its four forward edges (Eq. 2): none unless the two
+//   project   a thread per site: a_x = phi_x . r;
+//   brick     a CTA per brick of sites draws the words of block (x, t, 4, 0)
+//             and bonds the forward edges (Eq. 2): none unless the two
 //             projections have the same sign, else iff w < (1 - e^{-z}) 2^32
 //             with z = 4 kappa a_x a_y; the exponential is this file's own
 //             (range reduction and a Taylor polynomial with fused
-//             multiply-adds), so the decisions are reproducible bit for bit;
+//             multiply-adds), so the decisions are reproducible bit for bit.
+//             The brick's clusters are labelled in shared memory;
 //   unite     lock-free union-find over int32 parents (larger root under the
-//             smaller with atomicMin), so roots are the clusters' smallest
-//             sites;
-//   roots     every site points at its root; each root draws its flip
-//             (bit 31 of word 0 of block (root, t, 6, 0));
+//             smaller) of the bonds that leave a brick, so roots are the
+//             clusters' smallest sites;
+//   roots     every local root gets its cluster's root and the flip drawn for
+//             it (bit 31 of word 0 of block (root, t, 6, 0));
 //   reflect   every site of a flipped cluster is reflected in the hyperplane
 //             orthogonal to r (Eq. 3): phi <- phi - 2 (phi . r) r;
 //   observe   E = sum over the 4N edges of phi_x . phi_{x+mu} and M = sum of
-//             phi, reduced in binary64 (the summation order differs from a
-//             serial sum, so these agree with one to rounding only).
+//             phi, in fixed point or binary64 (the summation order differs
+//             from a serial sum, so these agree with one to rounding only).
 // Every operation that feeds a bond decision or a new field value is an
 // explicitly rounded intrinsic, so nothing is contracted differently from a
 // serial restatement compiled without contraction.
@@ -114,14 +114,16 @@ __device__ __forceinline__ uint32_t nb(uint32_t x, int mu, const Coords& k, uint
 // and w < (1 - e^{-z}) 2^32 with z = k4 q, all in binary64 with exp_neg.
 // GB300 runs binary64 at a small fraction of its binary32 rate, so a
 // binary32 estimate decides first, from the projections rounded to binary32
-// (af, each within 2^-24 relative): with both |af| >= 2^-60 the binary64
-// product is positive exactly when the signs agree, z in binary32 (three
-// roundings of 2^-24 and two products) is within 5 * 2^-24 relative, so
-// e^{-z} from expf (2 ulp) is within 40 * 5 * 2^-24 + 2^-22 of the binary64
-// value for z <= 40, and (1 - e) 2^32 is then within 2^16 of the binary64
-// threshold. A word more than 2^18 from the estimate takes the same decision
-// as the binary64 test; the others (about 1e-4 of the edges), edges with a
-// tiny projection and z near 40 take the binary64 test itself.
+// (af, each within 2^-24 relative): with both |af| >= 2^-60 the estimate of z
+// (three roundings of 2^-24 and two products) is within 5 * 2^-24 relative and
+// has the sign of q, so for 0 < z <= 40 e^{-z} from expf (2 ulp) is within
+// 40 * 5 * 2^-24 + 2^-22 of the binary64 value and (1 - e) 2^32 within 2^16 of
+// the binary64 threshold; beyond 40 both thresholds are 2^32 to binary32
+// precision, and for z < 0 the estimate is not positive. A word more than 2^18
+// from the estimate (words round to binary32 within 2^8) takes the same
+// decision as the binary64 test; the others (about 1e-4 of the edges), edges
+// with a tiny projection and estimates that are not a number take the
+// binary64 test itself.
 __device__ __forceinline__ bool bonded_exact(double ax, double ay, double k4, uint32_t w) {
   const double q = __dmul_rn(ax, ay);
   if (!(q > 0.0)) return false;
@@ -131,18 +133,9 @@ __device__ __forceinline__ bool bonded_exact(double ax, double ay, double k4, ui
 
 __device__ __forceinline__ bool bonded(const double* a, uint32_t x, uint32_t y, float fx, float fy, float k4f,
                                        double k4, uint32_t w) {
-  const float mx = fabsf(fx), my = fabsf(fy);
-  if (mx >= 0x1p-60f && my >= 0x1p-60f) {
-    if ((__float_as_uint(fx) ^ __float_as_uint(fy)) >> 31) return false;  // opposite signs: q < 0
-    const float zf = __fmul_rn(__fmul_rn(k4f, mx), my);
-    if (zf > 40.01f) return true;  // z > 40: e^{-z} is 0 in exp_neg, the threshold 2^32
-    if (zf < 39.99f) {
-      const float tf = __fmul_rn(__fsub_rn(1.0f, expf(-zf)), 0x1p32f);
-      const float wf = (float)w;  // within 2^8 of w
-      if (wf < tf - 0x1p18f) return true;
-      if (wf > tf + 0x1p18f) return false;
-    }
-  }
+  const float z = __fmul_rn(__fmul_rn(k4f, fx), fy);
+  const float d = __fsub_rn((float)w, __fmaf_rn(-expf(-z), 0x1p32f, 0x1p32f));  // w - (1 - e) 2^32
+  if (fabsf(d) > 0x1p18f && fminf(fabsf(fx), fabsf(fy)) >= 0x1p-60f) return d < 0.0f;
   return bonded_exact(a[x], a[y], k4, w);
 }
 
@@ -150,36 +143,60 @@ __device__ __forceinline__ double unit_interval(uint32_t w) {
   return __dsub_rn(__dmul_rn(__dadd_rn(__uint2double_rn(w), 0.5), 0x1p-31), 1.0);
 }
 
-__device__ int find_root(int* par, int x, int* err) {
-  for (int it = 0;; ++it) {
-    const int p = __ldcg(par + x);
-    if (p == x) return x;
-    const int gp = __ldcg(par + p);
-    if (gp == p) return p;
-    if (it >= kFindCap) {
-      atomicCAS(err, 0, 1);
-      return p;
-    }
-    atomicMin(par + x, gp);
-    x = gp;
-  }
+// Union-find over parents in global or shared memory: a link is one
+// compare-and-swap of a root's own entry, so only entries of non-roots change
+// otherwise, and halving a path is a plain store of an ancestor. G: global
+// memory (loads and stores past L1, which is not kept coherent).
+template <bool G>
+__device__ __forceinline__ int ld_par(const int* p) {
+  return G ? __ldcg(p) : *(const volatile int*)p;
+}
+template <bool G>
+__device__ __forceinline__ void st_par(int* p, int v) {
+  if (G) __stcg(p, v);
+  else *(volatile int*)p = v;
 }
 
-__device__ void unite(int* par, int a, int b, int* err) {
-  for (int it = 0; it < kUnionCap; ++it) {
-    a = find_root(par, a, err);
-    b = find_root(par, b, err);
-    if (a == b) return;
-    if (a < b) {
-      const int t = a;
-      a = b;
-      b = t;
+// The unions of a warp's list of n pairs, pair(k, a, b) giving the k-th. One
+// state machine per lane: a lane takes its next pair when its union is done,
+// and every warp-wide trip moves each busy lane one step (both nodes to their
+// grandparents, or at two distinct roots the larger hung under the smaller),
+// so lanes with long walks do not idle the others. Every lane of the warp
+// calls this.
+template <bool G, typename Pair>
+__device__ __forceinline__ void unite_list(int* par, int n, Pair pair, int* err) {
+  int k = threadIdx.x & 31, a = 0, b = 0;
+  bool busy = false;
+  for (int it = 0;; ++it) {
+    if (!busy && k < n) {
+      pair(k, a, b);
+      k += 32;
+      busy = true;
     }
-    const int old = atomicMin(par + a, b);
-    if (old == a) return;
-    a = old;
+    if (!__any_sync(0xffffffffu, busy)) return;
+    if (it >= kUnionCap) {
+      if (busy) atomicCAS(err, 0, 1);
+      return;
+    }
+    if (!busy) continue;
+    const int pa = ld_par<G>(par + a), pb = ld_par<G>(par + b);
+    if (pa == a && pb == b) {
+      if (a == b) {
+        busy = false;
+      } else {
+        const int hi = max(a, b), lo = min(a, b), old = atomicCAS(par + hi, hi, lo);
+        busy = old != hi;  // another lane hung that root first: go on from its parent
+        a = old;
+        b = lo;
+      }
+    } else {
+      const int ga = pa == a ? a : ld_par<G>(par + pa), gb = pb == b ? b : ld_par<G>(par + pb);
+      if (ga != pa) st_par<G>(par + a, ga);
+      if (gb != pb) st_par<G>(par + b, gb);
+      a = ga;
+      b = gb;
+    }
   }
-  atomicCAS(err, 0, 1);
 }
 
 #define GRID_LOOP(i, n) \
@@ -200,14 +217,13 @@ __device__ __forceinline__ uint32_t abs_high(double d) { return (uint32_t)__doub
 
 // The projections in binary64 and, for the bond kernel's first test, rounded
 // to binary32.
-__global__ void phi4_project_kernel(const F4* phi, double* a, float* af, int* par, int64_t n, Dir d, uint32_t* top) {
+__global__ void phi4_project_kernel(const F4* phi, double* a, float* af, int64_t n, Dir d, uint32_t* top) {
   uint32_t big = 0u;  // high word of the largest |component|
   GRID_LOOP(x, n) {
     const F4 f = phi[x];
     const double v = proj(f, d);
     a[x] = v;
     af[x] = __double2float_rn(v);
-    par[x] = (int)x;
     big = max(max(max(big, abs_high(f.x)), abs_high(f.y)), max(abs_high(f.z), abs_high(f.w)));
   }
   if (top) {
@@ -216,61 +232,245 @@ __global__ void phi4_project_kernel(const F4* phi, double* a, float* af, int* pa
   }
 }
 
-__global__ void phi4_bonds_kernel(const double* a, const float* af, uint8_t* bonds, int L, int64_t n, double k4,
-                                  uint32_t t, sw::KeySchedule ks) {
+// ------------------------------------------------------------ clusters
+//
+// Bonds and clusters brick by brick: a CTA takes a brick of B0 x B1 x B2 x B3
+// sites, decides the forward bonds of its sites and labels the brick's
+// clusters in shared memory; only the bonds that leave a brick (14 % of the
+// edges for 16 x 8 x 8 x 4) go to the union-find in global memory. With every
+// edge united in global memory (L = 64) the bonds ran 180 us, the unions 960
+// and the pass that points every site at its root 315, both waiting for
+// dependent L2 loads with 4 of 32 lanes active; the brick kernel runs 275 us,
+// bound by instruction issue (the Philox draws, expf and the walks), the unions
+// that are left 122 and the local roots' pass 75 to 97.
+//
+// Within a brick the local site order is the global one, so a component's
+// smallest local site is its smallest site. Results: par[x] = the smallest
+// site of x's brick component (its local root; itself for a local root), and
+// in bonds[x] the forward bonds that leave the brick (bits 0-3) and kLocalRoot
+// for a local root.
+constexpr uint32_t kLocalRoot = 16u;
+constexpr int kSiteMask = 0x7fffffff;  // a parent entry without its decision bit
+
+template <int B0, int B1, int B2, int B3, int NT>
+__global__ void __launch_bounds__(NT)
+    phi4_brick_kernel(const double* a, const float* af, uint8_t* bonds, int* par, int L, double k4, uint32_t t,
+                      sw::KeySchedule ks, int* err) {
+  constexpr int V = B0 * B1 * B2 * B3, S1 = B0, S2 = B0 * B1, S3 = B0 * B1 * B2;
+  __shared__ float s_af[V];
+  __shared__ int s_par[V];
+  __shared__ uint8_t s_b[V];  // bits 0-3: bonds inside the brick, 4-7: bonds that leave it
   const float k4f = __double2float_rn(k4);
-  GRID_LOOP(i, n) {
-    const uint32_t x = (uint32_t)i;
+  const uint32_t uL = (uint32_t)L, L2 = uL * uL, L3 = L2 * uL;
+  uint32_t q = blockIdx.x;
+  const uint32_t g0 = (uL + B0 - 1) / B0, g1 = (uL + B1 - 1) / B1, g2 = (uL + B2 - 1) / B2;
+  const uint32_t o0 = q % g0 * B0;
+  q /= g0;
+  const uint32_t o1 = q % g1 * B1;
+  q /= g1;
+  const uint32_t o2 = q % g2 * B2, o3 = q / g2 * B3;
+  const uint32_t base = o0 + uL * o1 + L2 * o2 + L3 * o3;
+  // the global site of local site l, and whether the lattice has it
+  auto site = [&](int l) {
+    return base + (uint32_t)(l % B0) + uL * (uint32_t)(l / S1 % B1) + L2 * (uint32_t)(l / S2 % B2) +
+           L3 * (uint32_t)(l / S3);
+  };
+  auto valid = [&](int l) {
+    return o0 + l % B0 < uL && o1 + l / S1 % B1 < uL && o2 + l / S2 % B2 < uL && o3 + l / S3 < uL;
+  };
+#pragma unroll 4
+  for (int l = threadIdx.x; l < V; l += NT) s_af[l] = valid(l) ? af[site(l)] : 0.0f;
+  __syncthreads();
+
+  for (int l = threadIdx.x; l < V; l += NT) {
+    uint32_t bits = 0u;
+    if (valid(l)) {
+      const uint32_t x = site(l);
+      const uint4 w4 = sw::philox4x32_10(make_uint4(x, t, 4u, 0u), ks);
+      const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+      const uint32_t i[4] = {(uint32_t)(l % B0), (uint32_t)(l / S1 % B1), (uint32_t)(l / S2 % B2), (uint32_t)(l / S3)};
+      const uint32_t o[4] = {o0, o1, o2, o3}, gs[4] = {1u, uL, L2, L3};
+      constexpr uint32_t B[4] = {B0, B1, B2, B3}, S[4] = {1, S1, S2, S3};
+      const float fx = s_af[l];
+#pragma unroll
+      for (int mu = 0; mu < 4; ++mu) {
+        const bool last = o[mu] + i[mu] + 1 == uL, inside = i[mu] + 1 < B[mu] && !last;
+        const uint32_t y = last ? x - (uL - 1) * gs[mu] : x + gs[mu];
+        const float fy = inside ? s_af[l + S[mu]] : af[y];
+        if (bonded(a, x, y, fx, fy, k4f, k4, w[mu])) bits |= (inside ? 1u : 16u) << mu;
+      }
+    }
+    s_b[l] = (uint8_t)bits;
+  }
+  __syncthreads();
+
+  // every site starts under the first site of its run of x0 bonds, and a bond
+  // in another direction is skipped when the one to its left joins the same
+  // two runs
+  for (int l = threadIdx.x; l < V; l += NT) {
+    int r = l;
+    while (r % B0 != 0 && (s_b[r - 1] & 1u)) --r;
+    s_par[l] = r;
+  }
+  __syncthreads();
+  {
+    // the warp's bonds to unite, as l + V (mu - 1), listed where the
+    // projections were (V / (NT / 32) words of two entries a warp)
+    constexpr int CAP = 2 * V / (NT / 32), J = V / NT;
+    static_assert(V % NT == 0 && 3 * V <= 65536 && CAP >= 2 * 32 * J, "list entries");
+    uint16_t* const list = reinterpret_cast<uint16_t*>(s_af) + (threadIdx.x >> 5) * CAP;
+    const int lane = threadIdx.x & 31;
+    int n = 0;
+    auto drain = [&] {
+      __syncwarp();
+      unite_list<false>(
+          s_par, n,
+          [&](int k, int& x, int& y) {
+            const int e = list[k], mu = e / V;
+            x = e - mu * V;
+            y = x + (mu == 0 ? S1 : mu == 1 ? S2 : S3);
+          },
+          err);
+      __syncwarp();
+      n = 0;
+    };
+#pragma unroll 1
+    for (int j = 0; j < J; ++j) {
+      const int l = threadIdx.x + j * NT;
+      const uint32_t b = s_b[l], left = l % B0 != 0 && (s_b[l - 1] & 1u) ? s_b[l - 1] : 0u;
+      constexpr int S[4] = {1, S1, S2, S3};
+#pragma unroll
+      for (int mu = 1; mu < 4; ++mu) {
+        const bool need = ((b >> mu) & 1u) && !(((left >> mu) & 1u) && (s_b[l - 1 + S[mu]] & 1u));
+        const uint32_t m = __ballot_sync(0xffffffffu, need);
+        if (need) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(l + V * (mu - 1));
+        n += __popc(m);
+      }
+      if (n > CAP - 96) drain();
+    }
+    if (n) drain();
+  }
+  __syncthreads();
+  for (int l = threadIdx.x; l < V; l += NT) {
+    if (!valid(l)) continue;
+    int r = l, p = s_par[r];
+    while (p != r) {
+      r = p;
+      p = s_par[r];
+    }
+    const uint32_t x = site(l);
+    par[x] = (int)site(r);
+    bonds[x] = (uint8_t)((s_b[l] >> 4) | (r == l ? kLocalRoot : 0u));
+  }
+}
+
+// Unions across brick borders, from the local roots of a bond's two sites;
+// consecutive sites whose bonds join the same two local roots unite once. A
+// warp lists the pairs of ROWS * 32 sites and unites them together: one site
+// in two has no bond that leaves its brick, and a union is a chain of
+// dependent L2 loads, so the lanes in flight set the rate. At L = 64 (bricks
+// of 16 x 8 x 8 x 4) eight rows take 122 us, four 130, two 134, one 177 and a
+// thread per site without lists 255; at L = 16 one row takes 12 us, two 12,
+// four 17 and eight 21 (fewer warps than the chip holds).
+constexpr int kUniteWarps = 4, kUniteCap = 2 * 128;
+template <int ROWS>
+__global__ void __launch_bounds__(32 * kUniteWarps)
+    phi4_unite_kernel(const uint8_t* bonds, int* par, int L, int64_t n, int* err) {
+  __shared__ int2 s_list[kUniteWarps][kUniteCap];
+  const int lane = threadIdx.x & 31;
+  int2* const list = s_list[threadIdx.x >> 5];
+  const int64_t x0 = ((int64_t)blockIdx.x * kUniteWarps + (threadIdx.x >> 5)) * (32 * ROWS);
+  uint32_t b[ROWS];
+#pragma unroll
+  for (int j = 0; j < ROWS; ++j) b[j] = x0 + 32 * j + lane < n ? bonds[x0 + 32 * j + lane] & 15u : 0u;
+  int cnt = 0;
+  auto drain = [&] {
+    __syncwarp();
+    unite_list<true>(
+        par, cnt,
+        [&](int k, int& u, int& v) {
+          u = list[k].x;
+          v = list[k].y;
+        },
+        err);
+    __syncwarp();
+    cnt = 0;
+  };
+#pragma unroll
+  for (int j = 0; j < ROWS; ++j) {
+    if (!__any_sync(0xffffffffu, b[j] != 0u)) continue;
+    const uint32_t x = (uint32_t)(x0 + 32 * j + lane);
     const Coords k = coords_of(x, (uint32_t)L);
-    const uint4 w4 = sw::philox4x32_10(make_uint4(x, t, 4u, 0u), ks);
-    const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
-    const float fx = af[x];
-    uint8_t b = 0;
+    const int ra = b[j] ? __ldcg(par + x) : -1;
+    int rb[4];
     uint32_t stride = 1;
 #pragma unroll
+    for (int mu = 0; mu < 4; ++mu, stride *= (uint32_t)L)
+      rb[mu] = (b[j] >> mu) & 1u ? __ldcg(par + nb(x, mu, k, (uint32_t)L, stride)) : -1;
+    const int la = __shfl_up_sync(0xffffffffu, ra, 1);
+#pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-      const uint32_t y = nb(x, mu, k, (uint32_t)L, stride);
-      if (bonded(a, x, y, fx, af[y], k4f, k4, w[mu])) b |= (uint8_t)(1u << mu);
-      stride *= (uint32_t)L;
+      const int lb = __shfl_up_sync(0xffffffffu, rb[mu], 1);
+      const bool need = rb[mu] >= 0 && ra != rb[mu] && !(lane > 0 && la == ra && lb == rb[mu]);
+      const uint32_t m = __ballot_sync(0xffffffffu, need);
+      if (need) list[cnt + __popc(m & ((1u << lane) - 1u))] = make_int2(ra, rb[mu]);
+      cnt += __popc(m);
     }
-    bonds[x] = b;
+    if (cnt > kUniteCap - 128) drain();
   }
+  if (cnt) drain();
 }
 
-__global__ void phi4_unite_kernel(const uint8_t* bonds, int* par, int L, int64_t n, int* err) {
-  GRID_LOOP(i, n) {
-    const uint32_t x = (uint32_t)i;
-    const uint8_t b = bonds[x];
-    if (!b) continue;
-    const Coords k = coords_of(x, (uint32_t)L);
-    uint32_t stride = 1;
-    for (int mu = 0; mu < 4; ++mu) {
-      if ((b >> mu) & 1u) unite(par, (int)x, (int)nb(x, mu, k, (uint32_t)L, stride), err);
-      stride *= (uint32_t)L;
-    }
+// Every local root gets its cluster's root and the decision drawn for it:
+// par[x] = root | decision << 31. Walks of other threads that meet a rewritten
+// entry still end at the same root. A warp lists the local roots of its
+// ROWS * 32 sites and takes them 32 at a time: four rows take 75 to 97 us at
+// L = 64 (eight 82 to 106, a thread per site 104 to 116); at L = 16 one row
+// takes 4.7 us and four 8.
+constexpr int kRootWarps = 4;
+template <int ROWS>
+__global__ void __launch_bounds__(32 * kRootWarps)
+    phi4_roots_kernel(const uint8_t* bonds, int* par, int64_t n, uint32_t t, sw::KeySchedule ks, int* err) {
+  __shared__ uint8_t s_list[kRootWarps][32 * ROWS];
+  static_assert(32 * ROWS <= 256, "8-bit entries");
+  const int lane = threadIdx.x & 31;
+  uint8_t* const list = s_list[threadIdx.x >> 5];
+  const int64_t x0 = ((int64_t)blockIdx.x * kRootWarps + (threadIdx.x >> 5)) * (32 * ROWS);
+  uint32_t b[ROWS];
+#pragma unroll
+  for (int j = 0; j < ROWS; ++j) b[j] = x0 + 32 * j + lane < n ? bonds[x0 + 32 * j + lane] : 0u;
+  int cnt = 0;
+#pragma unroll
+  for (int j = 0; j < ROWS; ++j) {
+    const bool is = (b[j] & kLocalRoot) != 0u;
+    const uint32_t m = __ballot_sync(0xffffffffu, is);
+    if (is) list[cnt + __popc(m & ((1u << lane) - 1u))] = (uint8_t)(32 * j + lane);
+    cnt += __popc(m);
   }
-}
-
-__global__ void phi4_roots_kernel(int* par, uint8_t* flip, int64_t n, uint32_t t, sw::KeySchedule ks, int* err) {
-  GRID_LOOP(x, n) {
-    int r = (int)x, p = __ldcg(par + r);
+  __syncwarp();
+  for (int k = lane; k < cnt; k += 32) {
+    const int x = (int)x0 + list[k];
+    int r = x, p = __ldcg(par + r) & kSiteMask;
     for (int it = 0; p != r; ++it) {
       if (it >= kFindCap) {
         atomicCAS(err, 0, 1);
         break;
       }
       r = p;
-      p = __ldcg(par + r);
+      p = __ldcg(par + r) & kSiteMask;
     }
-    par[x] = r;  // concurrent stores all write roots
-    if (r == (int)x) flip[x] = (uint8_t)(sw::philox4x32_10(make_uint4((uint32_t)x, t, 6u, 0u), ks).x >> 31);
+    const uint32_t f = sw::philox4x32_10(make_uint4((uint32_t)r, t, 6u, 0u), ks).x & 0x80000000u;
+    par[x] = (int)((uint32_t)r | f);
   }
 }
 
-__global__ void phi4_reflect_kernel(F4* phi, const double* a, const int* par, const uint8_t* flip, int64_t n,
-                                    Dir d) {
+__global__ void phi4_labels_kernel(const int* par, int* out, int64_t n) {
+  GRID_LOOP(x, n) out[x] = par[par[x] & kSiteMask] & kSiteMask;
+}
+
+__global__ void phi4_reflect_kernel(F4* phi, const double* a, const int* par, int64_t n, Dir d) {
   GRID_LOOP(x, n) {
-    if (!flip[par[x]]) continue;
+    if (par[par[x] & kSiteMask] >= 0) continue;  // the cluster's decision: not flipped
     const double m2a = __dmul_rn(-2.0, a[x]);
     F4 f = phi[x];
     f.x = __fma_rn(m2a, d.r[0], f.x);
@@ -379,6 +579,11 @@ constexpr int kObserveSteps = 16;
 // From 2^20 sites: below, the binary64 kernel takes 10 us or less (L = 16), most
 // of it latency, and the fixed-point one has too few blocks of sixteen slices.
 constexpr int64_t kObserveFixedSites = 1 << 20;
+// From 2^20 sites the large bricks (4096 sites: fewer bonds leave them) and the
+// merge with several rows a warp; below, one site a thread and small bricks, so
+// that L = 16 still has 256 CTAs: 8 us against 20 with 8 x 4 x 4 x 4 bricks of
+// 128 threads.
+constexpr int64_t kLargeSites = 1 << 20;
 
 __global__ void __launch_bounds__(kObserveThreads)
     phi4_observe_fixed_kernel(const F4* phi, int L, int64_t n, const uint32_t* top, int steps, double* out) {
@@ -478,7 +683,6 @@ struct sw_phi4 {
   float* af = nullptr;  // the projections rounded to binary32 (the bond kernel's first test)
   int* par = nullptr;
   uint8_t* bonds = nullptr;
-  uint8_t* flip = nullptr;
   double* obs = nullptr;  // [cap][5]: E, M0..M3
   uint32_t* top = nullptr;  // high word of the field's largest |component| (projection -> E and M)
   int* err = nullptr;
@@ -496,7 +700,7 @@ namespace {
   } while (0)
 
 void free_phi4(sw_phi4* h) {
-  void* ptrs[] = {h->phi, h->a, h->af, h->par, h->bonds, h->flip, h->obs, h->top, h->err};
+  void* ptrs[] = {h->phi, h->a, h->af, h->par, h->bonds, h->obs, h->top, h->err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -549,17 +753,37 @@ int direction(uint64_t seed, uint32_t t, double r[4]) {
   return -1;
 }
 
+template <int B0, int B1, int B2, int B3, int NT>
+void launch_brick(sw_phi4* h) {
+  const int L = h->L;
+  const unsigned g = (unsigned)((L + B0 - 1) / B0) * ((L + B1 - 1) / B1) * ((L + B2 - 1) / B2) * ((L + B3 - 1) / B3);
+  phi4_brick_kernel<B0, B1, B2, B3, NT>
+      <<<g, NT, 0, h->stream>>>(h->a, h->af, h->bonds, h->par, L, 4.0 * h->kappa, (uint32_t)h->t, h->ks, h->err);
+}
+
+template <int UNITE_ROWS, int ROOT_ROWS>
+void launch_merge(sw_phi4* h) {
+  const int64_t u = 32 * kUniteWarps * UNITE_ROWS, r = 32 * kRootWarps * ROOT_ROWS;
+  phi4_unite_kernel<UNITE_ROWS><<<(unsigned)((h->n + u - 1) / u), 32 * kUniteWarps, 0, h->stream>>>(
+      h->bonds, h->par, h->L, h->n, h->err);
+  phi4_roots_kernel<ROOT_ROWS><<<(unsigned)((h->n + r - 1) / r), 32 * kRootWarps, 0, h->stream>>>(
+      h->bonds, h->par, h->n, (uint32_t)h->t, h->ks, h->err);
+}
+
 // Direction, projections, bonds, clusters and flips of update t.
 int clusters(sw_phi4* h, Dir& d) {
   if (direction(h->seed, (uint32_t)h->t, d.r) != 0) return ffail(SW_EDEVICE, "no direction found");
   const int g = grid_of(h->n);
   uint32_t* const top = h->n >= kObserveFixedSites ? h->top : nullptr;
   if (top) F_CUDA(cudaMemsetAsync(top, 0, sizeof(uint32_t), h->stream), "range word");
-  phi4_project_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->af, h->par, h->n, d, top);
-  phi4_bonds_kernel<<<g, 256, 0, h->stream>>>(h->a, h->af, h->bonds, h->L, h->n, 4.0 * h->kappa, (uint32_t)h->t,
-                                              h->ks);
-  phi4_unite_kernel<<<g, 256, 0, h->stream>>>(h->bonds, h->par, h->L, h->n, h->err);
-  phi4_roots_kernel<<<g, 256, 0, h->stream>>>(h->par, h->flip, h->n, (uint32_t)h->t, h->ks, h->err);
+  phi4_project_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->af, h->n, d, top);
+  if (h->n >= kLargeSites) {
+    launch_brick<16, 8, 8, 4, 1024>(h);
+    launch_merge<8, 4>(h);
+  } else {
+    launch_brick<8, 4, 4, 2, 256>(h);
+    launch_merge<1, 1>(h);
+  }
   F_CUDA(cudaGetLastError(), "phi4 update launch");
   return SW_OK;
 }
@@ -605,7 +829,6 @@ int sw_phi4_create(int32_t L, double kappa, uint64_t seed, int32_t init, void* s
   if (e == cudaSuccess) e = cudaMalloc(&h->af, n * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&h->par, n * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->bonds, n);
-  if (e == cudaSuccess) e = cudaMalloc(&h->flip, n);
   if (e == cudaSuccess) e = cudaMalloc(&h->top, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&h->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int), h->stream);
@@ -641,7 +864,7 @@ int sw_phi4_sweep(sw_phi4* h, int32_t n) {
     if (rc != SW_OK) return rc;
     double* o = h->obs + 5 * (h->t - h->t_base);
     F_CUDA(cudaMemsetAsync(o, 0, 5 * sizeof(double), h->stream), "trace row");
-    phi4_reflect_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->par, h->flip, h->n, d);
+    phi4_reflect_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->par, h->n, d);
     if (h->n >= kObserveFixedSites) {
       const int V = h->L * h->L * h->L;
       const dim3 grid((V + kObserveThreads - 1) / kObserveThreads, (h->L + kObserveSteps - 1) / kObserveSteps);
@@ -705,10 +928,12 @@ int sw_phi4_labels(sw_phi4* h, int32_t* out, int32_t out_is_device) {
   Dir d;
   int rc = clusters(h, d);
   if (rc != SW_OK) return rc;
-  F_CUDA(cudaMemcpyAsync(out, h->par, (size_t)h->n * sizeof(int32_t),
-                         out_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream),
-         "labels copy");
+  // host labels pass through the projections' buffer (8 bytes a site), done with here
+  int32_t* const dst = out_is_device ? out : reinterpret_cast<int32_t*>(h->a);
+  phi4_labels_kernel<<<grid_of(h->n), 256, 0, h->stream>>>(h->par, dst, h->n);
+  F_CUDA(cudaGetLastError(), "phi4 labels launch");
   if (out_is_device) return SW_OK;
+  F_CUDA(cudaMemcpyAsync(out, dst, (size_t)h->n * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream), "labels copy");
   return check_phi4(h);
 }
 
