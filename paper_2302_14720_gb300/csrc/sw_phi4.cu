@@ -45,6 +45,7 @@ constexpr int kUnionCap = 1 << 16;
 
 struct Dir {
   double r[4];
+  double m2r[4];  // -2 r, exactly
 };
 
 // One site's field, binary64 x 4 (O1), 32-byte aligned.
@@ -215,6 +216,17 @@ __global__ void phi4_init_kernel(F4* phi, int64_t n, sw::KeySchedule ks, int col
 
 __device__ __forceinline__ uint32_t abs_high(double d) { return (uint32_t)__double2hiint(d) & 0x7fffffffu; }
 
+// v rounded to binary32, by integer operations where the result is a normal
+// number: the conversion instruction runs in the binary64 pipe, which bounds the
+// projection (four operations a site; 164 -> 156 us at L = 64 without it).
+__device__ __forceinline__ float to_binary32(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  if (((hi >> 20) & 0x7ffu) - 897u > 253u) return __double2float_rn(v);
+  const uint32_t m = __funnelshift_l(lo, hi, 3);  // low bits of the exponent, 23 bits of the mantissa
+  const uint32_t up = ((lo & 0x1fffffffu) + 0x0fffffffu + (m & 1u)) >> 29;  // to nearest, ties to even
+  return __uint_as_float((hi & 0x80000000u) | ((m - (896u << 23) + up) & 0x7fffffffu));
+}
+
 // The projections in binary64 and, for the bond kernel's first test, rounded
 // to binary32.
 __global__ void phi4_project_kernel(const F4* phi, double* a, float* af, int64_t n, Dir d, uint32_t* top) {
@@ -223,7 +235,7 @@ __global__ void phi4_project_kernel(const F4* phi, double* a, float* af, int64_t
     const F4 f = phi[x];
     const double v = proj(f, d);
     a[x] = v;
-    af[x] = __double2float_rn(v);
+    af[x] = to_binary32(v);
     big = max(max(max(big, abs_high(f.x)), abs_high(f.y)), max(abs_high(f.z), abs_high(f.w)));
   }
   if (top) {
@@ -471,12 +483,15 @@ __global__ void phi4_labels_kernel(const int* par, int* out, int64_t n) {
 __global__ void phi4_reflect_kernel(F4* phi, const double* a, const int* par, int64_t n, Dir d) {
   GRID_LOOP(x, n) {
     if (par[par[x] & kSiteMask] >= 0) continue;  // the cluster's decision: not flipped
-    const double m2a = __dmul_rn(-2.0, a[x]);
+    // a (-2 r_c) is the same product as (-2 a) r_c, both factors exact (unless
+    // -2 a overflows), and saves one of five binary64 operations: 171 -> 162 us
+    // at L = 64
+    const double ax = a[x];
     F4 f = phi[x];
-    f.x = __fma_rn(m2a, d.r[0], f.x);
-    f.y = __fma_rn(m2a, d.r[1], f.y);
-    f.z = __fma_rn(m2a, d.r[2], f.z);
-    f.w = __fma_rn(m2a, d.r[3], f.w);
+    f.x = __fma_rn(ax, d.m2r[0], f.x);
+    f.y = __fma_rn(ax, d.m2r[1], f.y);
+    f.z = __fma_rn(ax, d.m2r[2], f.z);
+    f.w = __fma_rn(ax, d.m2r[3], f.w);
     phi[x] = f;
   }
 }
@@ -576,24 +591,42 @@ __global__ void phi4_observe_kernel(const F4* phi, int L, int64_t n, double* out
 // are loaded and converted again: 2.25 conversions a site at L = 64.
 constexpr int kObserveThreads = 256;
 constexpr int kObserveSteps = 16;
-// From 2^20 sites: below, the binary64 kernel takes 10 us or less (L = 16), most
-// of it latency, and the fixed-point one has too few blocks of sixteen slices.
-constexpr int64_t kObserveFixedSites = 1 << 20;
 // From 2^20 sites the large bricks (4096 sites: fewer bonds leave them) and the
 // merge with several rows a warp; below, one site a thread and small bricks, so
 // that L = 16 still has 256 CTAs: 8 us against 20 with 8 x 4 x 4 x 4 bricks of
-// 128 threads.
+// 128 threads. E and M take the fixed-point kernel from there too: below, the
+// binary64 kernel takes 10 us or less (L = 16), most of it latency, and the
+// fixed-point one has too few blocks of sixteen slices.
 constexpr int64_t kLargeSites = 1 << 20;
 
+//
+// PROJECT: the same pass takes the projections of the next update, which read
+// the same field and are bound by the binary64 pipe while the sums are bound
+// by integer issue: 303 us together, 222 + 156 apart (L = 64).
+template <bool PROJECT>
 __global__ void __launch_bounds__(kObserveThreads)
-    phi4_observe_fixed_kernel(const F4* phi, int L, int64_t n, const uint32_t* top, int steps, double* out) {
+    phi4_observe_fixed_kernel(const F4* phi, int L, int64_t n, const uint32_t* top, int steps, double* out, double* a,
+                              float* af, Dir d, uint32_t* next_top) {
+  uint32_t big = 0u;
+  auto project = [&](const F4& f, size_t x) {
+    const double v = proj(f, d);
+    a[x] = v;
+    af[x] = __double2float_rn(v);
+    big = max(max(max(big, abs_high(f.x)), abs_high(f.y)), max(abs_high(f.z), abs_high(f.w)));
+  };
   const int et = (int)(*top >> 20);  // biased exponent of the largest component before the reflection
   if (et < 1023 - 400 || et > 1023 + 400) {
     // zero, subnormal, huge, infinite or NaN components: the binary64 sums
     double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    const int64_t b = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-    observe_binary64(phi, L, n, b * blockDim.x + threadIdx.x, (int64_t)gridDim.x * gridDim.y * blockDim.x, v);
+    const int64_t b = (int64_t)blockIdx.y * gridDim.x + blockIdx.x, x0 = b * blockDim.x + threadIdx.x,
+                  step = (int64_t)gridDim.x * gridDim.y * blockDim.x;
+    observe_binary64(phi, L, n, x0, step, v);
     block_add5(v, out);
+    if (PROJECT) {
+      for (int64_t x = x0; x < n; x += step) project(phi[x], x);
+      big = __reduce_max_sync(0xffffffffu, big);
+      if ((threadIdx.x & 31) == 0) atomicMax(next_top, big);
+    }
     return;
   }
   const int T = et - 1023 + 2;        // |phi| <= 2 max component < 2^T
@@ -607,10 +640,14 @@ __global__ void __launch_bounds__(kObserveThreads)
   const bool in0 = n0 - s0 < kObserveThreads, in1 = n1 - s0 < kObserveThreads;
   const int z0 = blockIdx.y * steps, z1 = min(z0 + steps, L);
   int64_t hh = 0, cr = 0, ll = 0, m[4] = {0, 0, 0, 0};
-  Fix4 own = to_fixed(phi[(size_t)z0 * V + sc], shift0);
+  const F4 first = phi[(size_t)z0 * V + sc];
+  if (PROJECT && have) project(first, (size_t)z0 * V + sc);
+  Fix4 own = to_fixed(first, shift0);
   for (int z = z0; z < z1; ++z) {
     const F4* slice = phi + (size_t)z * V;
-    const Fix4 up = to_fixed(phi[(size_t)(z + 1 == L ? 0 : z + 1) * V + sc], shift0);
+    const F4 fu = phi[(size_t)(z + 1 == L ? 0 : z + 1) * V + sc];
+    if (PROJECT && have && z + 1 < z1) project(fu, (size_t)(z + 1) * V + sc);
+    const Fix4 up = to_fixed(fu, shift0);
     const F4 g2 = slice[n2];
     longlong2(&buf)[2][kObserveThreads] = s_x[z & 1];
     buf[0][threadIdx.x] = make_longlong2(own.v[0], own.v[1]);
@@ -653,6 +690,10 @@ __global__ void __launch_bounds__(kObserveThreads)
     for (int c = 0; c < 4; ++c) v[1 + c] = (double)m[c] * u;
   }
   block_add5(v, out);
+  if (PROJECT) {
+    big = __reduce_max_sync(0xffffffffu, big);
+    if ((threadIdx.x & 31) == 0) atomicMax(next_top, big);
+  }
 }
 
 int grid_of(int64_t n) {
@@ -684,7 +725,7 @@ struct sw_phi4 {
   int* par = nullptr;
   uint8_t* bonds = nullptr;
   double* obs = nullptr;  // [cap][5]: E, M0..M3
-  uint32_t* top = nullptr;  // high word of the field's largest |component| (projection -> E and M)
+  uint32_t* top = nullptr;  // [2], by update parity: high word of the field's largest |component| (projection -> E and M)
   int* err = nullptr;
 };
 
@@ -737,7 +778,7 @@ int grow(sw_phi4* h, int64_t need) {
 }
 
 // O3 on the host: the first attempt k with 2^-20 < |v|^2 <= 1.
-int direction(uint64_t seed, uint32_t t, double r[4]) {
+int direction(uint64_t seed, uint32_t t, Dir& d) {
   const sw::KeySchedule ks = sw::make_key_schedule(seed);
   for (uint32_t k = 0; k < 1000; ++k) {
     const uint4 w = sw::philox4x32_10(make_uint4(k, t, 5u, 0u), ks);
@@ -746,7 +787,10 @@ int direction(uint64_t seed, uint32_t t, double r[4]) {
     const double s = std::fma(v[3], v[3], std::fma(v[2], v[2], std::fma(v[1], v[1], v[0] * v[0])));
     if (s <= 1.0 && s > 0x1p-20) {
       const double nrm = std::sqrt(s);
-      for (int a = 0; a < 4; ++a) r[a] = v[a] / nrm;
+      for (int a = 0; a < 4; ++a) {
+        d.r[a] = v[a] / nrm;
+        d.m2r[a] = -2.0 * d.r[a];
+      }
       return 0;
     }
   }
@@ -770,13 +814,21 @@ void launch_merge(sw_phi4* h) {
       h->bonds, h->par, h->n, (uint32_t)h->t, h->ks, h->err);
 }
 
-// Direction, projections, bonds, clusters and flips of update t.
-int clusters(sw_phi4* h, Dir& d) {
-  if (direction(h->seed, (uint32_t)h->t, d.r) != 0) return ffail(SW_EDEVICE, "no direction found");
-  const int g = grid_of(h->n);
-  uint32_t* const top = h->n >= kObserveFixedSites ? h->top : nullptr;
-  if (top) F_CUDA(cudaMemsetAsync(top, 0, sizeof(uint32_t), h->stream), "range word");
-  phi4_project_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->af, h->n, d, top);
+// The direction of update t and, on large lattices, its cleared range word.
+int begin_update(sw_phi4* h, int64_t t, Dir& d) {
+  if (direction(h->seed, (uint32_t)t, d) != 0) return ffail(SW_EDEVICE, "no direction found");
+  if (h->n >= kLargeSites) F_CUDA(cudaMemsetAsync(h->top + (t & 1), 0, sizeof(uint32_t), h->stream), "range word");
+  return SW_OK;
+}
+
+// Projections of update t on direction d.
+void project(sw_phi4* h, const Dir& d) {
+  phi4_project_kernel<<<grid_of(h->n), 256, 0, h->stream>>>(h->phi, h->a, h->af, h->n, d,
+                                                            h->n >= kLargeSites ? h->top + (h->t & 1) : nullptr);
+}
+
+// Bonds, clusters and flips of update t from its projections.
+int clusters(sw_phi4* h) {
   if (h->n >= kLargeSites) {
     launch_brick<16, 8, 8, 4, 1024>(h);
     launch_merge<8, 4>(h);
@@ -794,7 +846,9 @@ extern "C" {
 
 int sw_phi4_direction(uint64_t seed, uint32_t t, double* r_out) {
   if (!r_out) return ffail(SW_EINVAL, "NULL argument");
-  if (direction(seed, t, r_out) != 0) return ffail(SW_EDEVICE, "no direction found");
+  Dir d;
+  if (direction(seed, t, d) != 0) return ffail(SW_EDEVICE, "no direction found");
+  for (int a = 0; a < 4; ++a) r_out[a] = d.r[a];
   return SW_OK;
 }
 
@@ -829,7 +883,7 @@ int sw_phi4_create(int32_t L, double kappa, uint64_t seed, int32_t init, void* s
   if (e == cudaSuccess) e = cudaMalloc(&h->af, n * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&h->par, n * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->bonds, n);
-  if (e == cudaSuccess) e = cudaMalloc(&h->top, sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&h->top, 2 * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&h->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int), h->stream);
   if (e == cudaSuccess) {
@@ -857,23 +911,41 @@ int sw_phi4_sweep(sw_phi4* h, int32_t n) {
   if (n < 0) return ffail(SW_EINVAL, "n must be >= 0");
   int rc = grow(h, h->t - h->t_base + n);
   if (rc != SW_OK) return rc;
-  const int g = grid_of(h->n);
+  if (n == 0) return SW_OK;
+  const int g = grid_of(h->n), L = h->L;
+  const bool large = h->n >= kLargeSites;
+  const dim3 og((unsigned)(((int64_t)L * L * L + kObserveThreads - 1) / kObserveThreads),
+                (unsigned)((L + kObserveSteps - 1) / kObserveSteps));
+  Dir d, next{};
+  rc = begin_update(h, h->t, d);
+  if (rc != SW_OK) return rc;
+  project(h, d);
   for (int32_t k = 0; k < n; ++k) {
-    Dir d;
-    rc = clusters(h, d);
+    rc = clusters(h);
     if (rc != SW_OK) return rc;
     double* o = h->obs + 5 * (h->t - h->t_base);
+    uint32_t* const top = h->top + (h->t & 1);
     F_CUDA(cudaMemsetAsync(o, 0, 5 * sizeof(double), h->stream), "trace row");
     phi4_reflect_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->par, h->n, d);
-    if (h->n >= kObserveFixedSites) {
-      const int V = h->L * h->L * h->L;
-      const dim3 grid((V + kObserveThreads - 1) / kObserveThreads, (h->L + kObserveSteps - 1) / kObserveSteps);
-      phi4_observe_fixed_kernel<<<grid, kObserveThreads, 0, h->stream>>>(h->phi, h->L, h->n, h->top, kObserveSteps, o);
-    } else {
-      phi4_observe_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->L, h->n, o);
+    // E and M, with the next update's projections unless the call ends here
+    // (the caller may change the field before the next one)
+    const bool more = k + 1 < n;
+    if (more) {
+      rc = begin_update(h, h->t + 1, next);
+      if (rc != SW_OK) return rc;
     }
+    if (large && more)
+      phi4_observe_fixed_kernel<true><<<og, kObserveThreads, 0, h->stream>>>(
+          h->phi, L, h->n, top, kObserveSteps, o, h->a, h->af, next, h->top + ((h->t + 1) & 1));
+    else if (large)
+      phi4_observe_fixed_kernel<false>
+          <<<og, kObserveThreads, 0, h->stream>>>(h->phi, L, h->n, top, kObserveSteps, o, nullptr, nullptr, d, nullptr);
+    else
+      phi4_observe_kernel<<<g, 256, 0, h->stream>>>(h->phi, L, h->n, o);
     F_CUDA(cudaGetLastError(), "phi4 reflect launch");
     h->t += 1;
+    if (more && !large) project(h, next);
+    d = next;
   }
   return SW_OK;
 }
@@ -926,7 +998,10 @@ int sw_phi4_set_field(sw_phi4* h, const double* in, uint32_t t, int32_t in_is_de
 int sw_phi4_labels(sw_phi4* h, int32_t* out, int32_t out_is_device) {
   if (!h || !out) return ffail(SW_EINVAL, "NULL argument");
   Dir d;
-  int rc = clusters(h, d);
+  int rc = begin_update(h, h->t, d);
+  if (rc != SW_OK) return rc;
+  project(h, d);
+  rc = clusters(h);
   if (rc != SW_OK) return rc;
   // host labels pass through the projections' buffer (8 bytes a site), done with here
   int32_t* const dst = out_is_device ? out : reinterpret_cast<int32_t*>(h->a);
