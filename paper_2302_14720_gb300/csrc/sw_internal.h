@@ -193,6 +193,7 @@ cudaError_t launch_export_bonds(int shape, const SweepArgs& a, uint8_t* out, cud
 // border cluster's new state into tb.nval, and phase 3 assigns the states and
 // sums E, M. Labels come from launch_phase3's labels mode. a.q >= 2.
 constexpr int kPottsShape = 6;
+constexpr int kPottsPad = 64;  // bytes of the state buffer past its last site (phase 1 loads whole row words)
 cudaError_t launch_potts_phase1(const SweepArgs& a, cudaStream_t st);
 cudaError_t launch_potts_phase3(const SweepArgs& a, cudaStream_t st);
 

@@ -71,69 +71,130 @@ __device__ __forceinline__ uint32_t spin_bytes4(uint32_t nib) {
   return 0x01010101u | (spread * 0xFEu);
 }
 
+// Sign bits of the 16 spins of one 16-byte load.
+__device__ __forceinline__ uint32_t sign_bits16(uint4 u) {
+  return sign_bits4(u.x) | (sign_bits4(u.y) << 4) | (sign_bits4(u.z) << 8) | (sign_bits4(u.w) << 12);
+}
+
+// Sign bits of the nb <= 32 spins from p on; n spins from `all` on are the
+// whole lattice. On aligned rows two 16-byte loads; else the two or three
+// 16-byte windows that the word straddles, shifted into place (a lattice
+// whose side is not a multiple of 16 has one row in 16 aligned). Only a word
+// whose windows would leave the lattice's memory, at its two ends, goes byte
+// by byte. (With byte loads and stores, each lane on a sector of its own, and
+// a Philox block a site, L = 8191 took 748 us a sweep; with these loads,
+// store_rows4 and bond_draws' 17th block 447 us, where L = 8192 takes 385.)
 // Spins are loaded past L1 (ld.cg): other CTAs of the fused batch kernel
 // write them earlier in the same launch, and L1 is not kept coherent.
-__device__ __forceinline__ uint32_t load_spin_bits(const int8_t* p, int nb, bool vec) {
+__device__ __forceinline__ uint32_t load_spin_bits(const int8_t* p, int nb, bool vec, const int8_t* all, int64_t n) {
   if (vec && nb == 32) {
     const uint4* q = reinterpret_cast<const uint4*>(p);
     const uint4 u = __ldcg(q), v = __ldcg(q + 1);
-    return sign_bits4(u.x) | (sign_bits4(u.y) << 4) | (sign_bits4(u.z) << 8) | (sign_bits4(u.w) << 12) |
-           (sign_bits4(v.x) << 16) | (sign_bits4(v.y) << 20) | (sign_bits4(v.z) << 24) |
-           (sign_bits4(v.w) << 28);
+    return sign_bits16(u) | (sign_bits16(v) << 16);
+  }
+  const int off = (int)(reinterpret_cast<uintptr_t>(p) & 15u), nwin = (off + nb + 15) >> 4;
+  const int8_t* w0 = p - off;
+  const uint32_t valid = 0xffffffffu >> (32 - nb);
+  if (w0 >= all && w0 + 16 * nwin <= all + n) {
+    const uint4* q = reinterpret_cast<const uint4*>(w0);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const uint4 u = __ldcg(q), v = nwin > 1 ? __ldcg(q + 1) : zero, x = nwin > 2 ? __ldcg(q + 2) : zero;
+    return __funnelshift_r(sign_bits16(u) | (sign_bits16(v) << 16), sign_bits16(x), off) & valid;
   }
   uint32_t bits = 0;
   for (int k = 0; k < nb; ++k) bits |= (uint32_t)(__ldcg(p + k) < 0) << k;
   return bits;
 }
 
-__device__ __forceinline__ void store_spin_bits(int8_t* p, uint32_t bits, int nb, bool vec) {
-  if (vec && nb == 32) {
-    uint4 u, v;
-    u.x = spin_bytes4(bits & 0xFu);
-    u.y = spin_bytes4((bits >> 4) & 0xFu);
-    u.z = spin_bytes4((bits >> 8) & 0xFu);
-    u.w = spin_bytes4((bits >> 12) & 0xFu);
-    v.x = spin_bytes4((bits >> 16) & 0xFu);
-    v.y = spin_bytes4((bits >> 20) & 0xFu);
-    v.z = spin_bytes4((bits >> 24) & 0xFu);
-    v.w = spin_bytes4(bits >> 28);
-    uint4* q = reinterpret_cast<uint4*>(p);
-    q[0] = u;
-    q[1] = v;
-    return;
+// 32 spins to 16-byte aligned memory.
+__device__ __forceinline__ void store_spin_bits(int8_t* p, uint32_t bits) {
+  uint4 u, v;
+  u.x = spin_bytes4(bits & 0xFu);
+  u.y = spin_bytes4((bits >> 4) & 0xFu);
+  u.z = spin_bytes4((bits >> 8) & 0xFu);
+  u.w = spin_bytes4((bits >> 12) & 0xFu);
+  v.x = spin_bytes4((bits >> 16) & 0xFu);
+  v.y = spin_bytes4((bits >> 20) & 0xFu);
+  v.z = spin_bytes4((bits >> 24) & 0xFu);
+  v.w = spin_bytes4(bits >> 28);
+  uint4* q = reinterpret_cast<uint4*>(p);
+  q[0] = u;
+  q[1] = v;
+}
+
+// A tile's rows to memory of any alignment by the whole block, as 4-byte
+// words on 4-byte boundaries: `first` is where column 0 of row 0 goes, rows
+// lie `pitch` bytes apart, and bytes4(y, x) gives the bytes of columns
+// x .. x + 3 of row y, x > -4 (the columns outside [0, ncols) are not
+// stored). Word c of a row starts (4 c - row address mod 4) columns from its
+// first; only the row's first and last word, shared with the neighbour tiles
+// or rows, may go byte by byte.
+template <int TW, int NT, typename F>
+__device__ __forceinline__ void store_rows4(int8_t* first, int64_t pitch, int nrows, int ncols, F bytes4) {
+  constexpr int G = TW / 4 + 1;
+  for (int i = threadIdx.x; i < nrows * G; i += NT) {
+    const int y = i / G, c = i - y * G;
+    int8_t* row = first + y * pitch;
+    const int x = 4 * c - (int)(reinterpret_cast<uintptr_t>(row) & 3u);
+    if (x >= ncols) continue;
+    const uint32_t v = bytes4(y, x);
+    if (x >= 0 && x + 4 <= ncols) {
+      *reinterpret_cast<uint32_t*>(row + x) = v;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (x + k >= 0 && x + k < ncols) row[x + k] = (int8_t)(v >> (8 * k));
+    }
   }
-  for (int k = 0; k < nb; ++k) p[k] = ((bits >> k) & 1u) ? (int8_t)-1 : (int8_t)1;
+}
+
+// The states of 36 sites from p on as nine 32-bit words, from the ten 4-byte
+// boundaries around them.
+__device__ __forceinline__ void load_states36(const int8_t* p, uint32_t (&A)[9]) {
+  const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 3u);
+  const uint32_t* q = reinterpret_cast<const uint32_t*>(p - off);
+  uint32_t w = q[0];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const uint32_t next = q[k + 1];
+    A[k] = __funnelshift_r(w, next, 8 * off);
+    w = next;
+  }
 }
 
 // §6 (q-state Potts): bit b of eqE / eqS is set iff site x0 + b of `row`
 // has the same state as its east neighbour (column x0 + b + 1 mod L) / as
-// the site below it (`rowS`, the next row mod L); nb valid columns. A whole
-// 16-byte aligned word compares four states per instruction.
+// the site below it (`rowS`, the next row mod L), for the nb valid columns
+// (the caller masks the others). Four states are compared per instruction.
+// ALIGNED (L is a multiple of 16): 16-byte loads; else 4-byte words shifted
+// into place (with three byte loads a site and byte stores L = 8191 took 671
+// us a sweep, 532 so). Loads may reach kPottsPad bytes past the
+// lattice: the library's own buffer is that much longer. The two forms are
+// kernels of their own: one kernel with both cost aligned lattices 2 %.
+template <bool ALIGNED>
 __device__ __forceinline__ void potts_equal_bits(const int8_t* row, const int8_t* rowS, int x0, int nb, int L,
-                                                 bool vec, uint32_t& eqE, uint32_t& eqS) {
-  if (vec && nb == 32) {
+                                                 uint32_t& eqE, uint32_t& eqS) {
+  uint32_t A[9], B[9];
+  if (ALIGNED) {
     const uint4 a0 = *reinterpret_cast<const uint4*>(row + x0), a1 = *reinterpret_cast<const uint4*>(row + x0 + 16);
     const uint4 b0 = *reinterpret_cast<const uint4*>(rowS + x0), b1 = *reinterpret_cast<const uint4*>(rowS + x0 + 16);
-    const uint32_t A[9] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w,
-                           (uint32_t)(uint8_t)row[x0 + 32 == L ? 0 : x0 + 32]};
-    const uint32_t B[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-    uint32_t e = 0u, d = 0u;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      // the four east neighbours of word k's states: bytes 1-3 of word k, byte 0 of word k + 1
-      e |= sign_bits4(__vcmpeq4(A[k], __funnelshift_r(A[k], A[k + 1], 8))) << (4 * k);
-      d |= sign_bits4(__vcmpeq4(A[k], B[k])) << (4 * k);
-    }
-    eqE = e;
-    eqS = d;
-    return;
+    A[0] = a0.x, A[1] = a0.y, A[2] = a0.z, A[3] = a0.w, A[4] = a1.x, A[5] = a1.y, A[6] = a1.z, A[7] = a1.w;
+    B[0] = b0.x, B[1] = b0.y, B[2] = b0.z, B[3] = b0.w, B[4] = b1.x, B[5] = b1.y, B[6] = b1.z, B[7] = b1.w;
+    A[8] = (uint32_t)(uint8_t)row[x0 + 32 >= L ? 0 : x0 + 32];
+  } else {
+    load_states36(row + x0, A);
+    load_states36(rowS + x0, B);
   }
   uint32_t e = 0u, d = 0u;
-  for (int b = 0; b < nb; ++b) {
-    const int x = x0 + b;
-    const int8_t v = row[x];
-    e |= (uint32_t)(v == row[x + 1 == L ? 0 : x + 1]) << b;
-    d |= (uint32_t)(v == rowS[x]) << b;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    // the four east neighbours of word k's states: bytes 1-3 of word k, byte 0 of word k + 1
+    e |= sign_bits4(__vcmpeq4(A[k], __funnelshift_r(A[k], A[k + 1], 8))) << (4 * k);
+    d |= sign_bits4(__vcmpeq4(A[k], B[k])) << (4 * k);
+  }
+  if (x0 + nb == L && !(ALIGNED && nb == 32)) {  // the last column's east neighbour is column 0
+    const uint32_t last = 1u << (nb - 1);
+    e = row[L - 1] == row[0] ? e | last : e & ~last;
   }
   eqE = e;
   eqS = d;
@@ -510,53 +571,46 @@ __device__ __forceinline__ bool cta_args(const SweepArgs& a0, const BatchArgs& b
 
 // ================================================================ phase 1
 
-// The bond draws (C5) of the row word of sites i0 .. i0 + nb - 1 in sweep t:
-// bit b of .x (.y) is set iff the east (south) word of site i0 + b is below
-// thr. Site i takes words x0 (east) and x1 (south) of block (i >> 1, t, 0, 0)
-// when i is even, x2 and x3 when it is odd.
-__device__ __forceinline__ uint2 bond_draws(uint32_t i0, int nb, int L, uint32_t t, uint32_t thr,
-                                            const KeySchedule& ks) {
+// Push the draws of block q, two sites, into the masks: each comparison is
+// the carry of one subtraction, added in as the new lowest bit (a set carry:
+// word >= thr, no bond). Fewer integer-pipe operations than a compare and a
+// select each.
+__device__ __forceinline__ void push_draws(uint32_t& rE, uint32_t& rS, const uint4& q, uint32_t thr) {
+  asm("{\n\t.reg .u32 d;\n\t"
+      "sub.cc.u32 d, %2, %6;\n\taddc.u32 %0, %0, %0;\n\t"
+      "sub.cc.u32 d, %4, %6;\n\taddc.u32 %0, %0, %0;\n\t"
+      "sub.cc.u32 d, %3, %6;\n\taddc.u32 %1, %1, %1;\n\t"
+      "sub.cc.u32 d, %5, %6;\n\taddc.u32 %1, %1, %1;\n\t}"
+      : "+r"(rE), "+r"(rS)
+      : "r"(q.x), "r"(q.y), "r"(q.z), "r"(q.w), "r"(thr));
+}
+
+// The bond draws (C5) of the 32 sites from i0 on in sweep t: bit b of .x
+// (.y) is set iff the east (south) word of site i0 + b is below thr. Site i
+// takes words x0 (east) and x1 (south) of block (i >> 1, t, 0, 0) when i is
+// even, x2 and x3 when it is odd; the first site pushed ends at bit 31, so
+// one bit reversal and a complement finish the masks. From an odd i0 (rows of
+// an odd side) the 16 blocks start one site early and the first site of a
+// 17th pushes that one out (a block a site, the straightforward form: phase 2
+// and resolve with draws 211 us at L = 8191, 123 us so). Words cut by the lattice's edge are drawn
+// whole (the caller masks them): their lanes share a warp with whole words
+// and would take it through a second loop.
+__device__ __forceinline__ uint2 bond_draws(uint32_t i0, int L, uint32_t t, uint32_t thr, const KeySchedule& ks) {
   uint32_t rE = 0u, rS = 0u;
+  const uint32_t p0 = i0 >> 1;
   if ((L & 1) == 0) {
-    // even L: sites i0+b, i0+b+1 (b even) share Philox block (i0+b)/2
-    if (nb == 32) {
-      // a whole word: each comparison is the carry of one subtraction, added
-      // into the mask as its new lowest bit (a set carry: q >= thr, no bond),
-      // so site 0 ends at bit 31; one bit reversal and a complement at the
-      // end. Fewer integer-pipe operations than a compare and a select each.
 #pragma unroll 4
-      for (int b = 0; b < 32; b += 2) {
-        const uint4 q = philox4x32_10(make_uint4((i0 + b) >> 1, t, 0u, 0u), ks);
-        asm("{\n\t.reg .u32 d;\n\t"
-            "sub.cc.u32 d, %2, %6;\n\taddc.u32 %0, %0, %0;\n\t"
-            "sub.cc.u32 d, %4, %6;\n\taddc.u32 %0, %0, %0;\n\t"
-            "sub.cc.u32 d, %3, %6;\n\taddc.u32 %1, %1, %1;\n\t"
-            "sub.cc.u32 d, %5, %6;\n\taddc.u32 %1, %1, %1;\n\t}"
-            : "+r"(rE), "+r"(rS)
-            : "r"(q.x), "r"(q.y), "r"(q.z), "r"(q.w), "r"(thr));
-      }
-      rE = __brev(~rE);
-      rS = __brev(~rS);
-    } else {
-#pragma unroll 4
-      for (int b = 0; b < 32; b += 2) {
-        if (b < nb) {
-          const uint4 q = philox4x32_10(make_uint4((i0 + b) >> 1, t, 0u, 0u), ks);
-          rE |= ((uint32_t)(q.x < thr) << b) | ((uint32_t)(q.z < thr) << (b + 1));
-          rS |= ((uint32_t)(q.y < thr) << b) | ((uint32_t)(q.w < thr) << (b + 1));
-        }
-      }
-    }
+    for (int b = 0; b < 16; ++b) push_draws(rE, rS, philox4x32_10(make_uint4(p0 + b, t, 0u, 0u), ks), thr);
   } else {
-    for (int b = 0; b < nb; ++b) {
-      const uint32_t i = i0 + b;
-      const uint4 q = philox4x32_10(make_uint4(i >> 1, t, 0u, 0u), ks);
-      const uint32_t we = (i & 1u) ? q.z : q.x, ws = (i & 1u) ? q.w : q.y;
-      rE |= (uint32_t)(we < thr) << b;
-      rS |= (uint32_t)(ws < thr) << b;
+#pragma unroll 2
+    for (int b = 0; b < 16; ++b) push_draws(rE, rS, philox4x32_10(make_uint4(p0 + b, t, 0u, 0u), ks), thr);
+    if (i0 & 1u) {
+      const uint4 q = philox4x32_10(make_uint4(p0 + 16, t, 0u, 0u), ks);
+      rE = 2u * rE + (uint32_t)(q.x >= thr);
+      rS = 2u * rS + (uint32_t)(q.y >= thr);
     }
   }
-  return make_uint2(rE, rS);
+  return make_uint2(__brev(~rE), __brev(~rS));
 }
 
 // Phase 1 runs one warp per 32-column band and asks for 1280 resident
@@ -617,10 +671,13 @@ struct P1Shared {
 
 // SPINS_GIVEN: the caller has put the spin words in S.sd[0] and the halo's
 // spins in S.bb (east column, south row), as phase 3 of the previous sweep
-// leaves them (phase31_kernel); the spins are not read from global memory.
+// leaves them (phase31_kernel); the spins are not read from global memory,
+// and the draws are in a.draws_in (taken by the merge before that launch).
 // POTTS: spins_in holds q-state Potts states (§6); an edge may bond iff its
-// two states are equal, and no spin words or halo spins are kept.
-template <int WPR, int TH, int H, bool BATCH, bool SPINS_GIVEN = false, bool POTTS = false>
+// two states are equal, and no spin words or halo spins are kept; ALIGNED as
+// in potts_equal_bits.
+template <int WPR, int TH, int H, bool BATCH, bool SPINS_GIVEN = false, bool POTTS = false,
+          bool ALIGNED = false>
 __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const SweepArgs& a0, const BatchArgs& bat,
                                             int T, int k) {
   using Tl = Tile<WPR, TH, H>;
@@ -667,7 +724,8 @@ __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const Sweep
       const int nbw = max(0, min(32, P.ncols - 32 * w));
       uint32_t sb = 0u;
       if (y < P.nrows && nbw)
-        sb = load_spin_bits(a.spins_in + (size_t)(P.y0 + y) * L + P.x0 + 32 * w, nbw, g.aligned16);
+        sb = load_spin_bits(a.spins_in + (size_t)(P.y0 + y) * L + P.x0 + 32 * w, nbw, g.aligned16, a.spins_in,
+                            (int64_t)L * L);
       s_spin[y][w] = sb;
     }
     __syncthreads();
@@ -683,7 +741,9 @@ __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const Sweep
     }
     for (int ww = tid; ww < WPR; ww += NT) {
       const int nbw = max(0, min(32, P.ncols - 32 * ww));
-      hS[ww] = nbw ? load_spin_bits(a.spins_in + (size_t)ys * L + P.x0 + 32 * ww, nbw, g.aligned16) : 0u;
+      hS[ww] = nbw ? load_spin_bits(a.spins_in + (size_t)ys * L + P.x0 + 32 * ww, nbw, g.aligned16, a.spins_in,
+                                    (int64_t)L * L)
+                   : 0u;
     }
     __syncthreads();
   }
@@ -700,8 +760,8 @@ __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const Sweep
     if (POTTS) {
       if (vmask) {
         const int yg = P.y0 + y;
-        potts_equal_bits(a.spins_in + (size_t)yg * L, a.spins_in + (size_t)(yg + 1 == L ? 0 : yg + 1) * L,
-                         P.x0 + 32 * w, nb, L, g.aligned16, eqE, eqS);
+        potts_equal_bits<ALIGNED>(a.spins_in + (size_t)yg * L, a.spins_in + (size_t)(yg + 1 == L ? 0 : yg + 1) * L,
+                         P.x0 + 32 * w, nb, L, eqE, eqS);
         eqE &= vmask;
         eqS &= vmask;
       }
@@ -720,13 +780,13 @@ __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const Sweep
     }
     uint32_t rE = 0, rS = 0;
     if (vmask) {
-      if (a.draws_in) {
+      if (SPINS_GIVEN || a.draws_in) {
         const uint2 d = __ldcs(a.draws_in + (size_t)P.tile * RW + rw);
         rE = d.x;
         rS = d.y;
       } else {
-        const uint2 d = bond_draws((uint32_t)(P.y0 + y) * (uint32_t)L + (uint32_t)(P.x0 + 32 * w), nb, L, a.t,
-                                   a.thr, a.ks);
+        const uint2 d =
+            bond_draws((uint32_t)(P.y0 + y) * (uint32_t)L + (uint32_t)(P.x0 + 32 * w), L, a.t, a.thr, a.ks);
         rE = d.x;
         rS = d.y;
       }
@@ -1076,14 +1136,22 @@ __device__ __forceinline__ void draw_next_bonds(const SweepArgs& a, int tile, in
     const int nb = max(0, min(32, P.ncols - 32 * w));
     if (y < P.nrows && nb > 0)
       __stcs(a.draws_out + (size_t)tile * RW + rw,
-             bond_draws((uint32_t)(P.y0 + y) * (uint32_t)L + (uint32_t)(P.x0 + 32 * w), nb, L, a.t + 1u, a.thr, a.ks));
+             bond_draws((uint32_t)(P.y0 + y) * (uint32_t)L + (uint32_t)(P.x0 + 32 * w), L, a.t + 1u, a.thr,
+                        a.ks));
   }
 }
 
 // With a.draws_out the block has kDrawWarps more warps than edges (TH + TW
-// threads); they draw the first draw_split row words of the tile.
+// threads); they draw the first draw_split row words of the tile. The merge
+// hides the latency of its walks by warps in flight, so the draws may not
+// raise the registers above those of a full SM (39 a thread instead of 32:
+// phase 2 + resolve at L = 8192 53 -> 62 us).
+template <int TH, int TW>
+constexpr int phase2_threads() {
+  return TH + TW + 32 * kDrawWarps;
+}
 template <int WPR, int TH, int H, bool BATCH>
-__global__ void phase2_kernel(const SweepArgs a0, const BatchArgs bat) {
+__global__ void __launch_bounds__(phase2_threads<TH, 32 * WPR>(), 2048 / phase2_threads<TH, 32 * WPR>()) phase2_kernel(const SweepArgs a0, const BatchArgs bat) {
   using Tl = Tile<WPR, TH, H>;
   if (!BATCH && a0.draws_out && threadIdx.x >= TH + Tl::TW) {
     draw_next_bonds<WPR, TH, H>(a0, blockIdx.x, threadIdx.x - (TH + Tl::TW), 0, draw_split<Tl::RW>());
@@ -1144,7 +1212,7 @@ __device__ __forceinline__ void resolve_body(const SweepArgs& a0, const BatchArg
 // kDrawWarps more warps draw the tile's row words from draw_split on.
 constexpr int kResolveThreads = 128;
 template <int WPR, int TH, int H, bool BATCH>
-__global__ void resolve_kernel(const SweepArgs a0, const BatchArgs bat) {
+__global__ void __launch_bounds__(kResolveThreads + 32 * kDrawWarps, 10) resolve_kernel(const SweepArgs a0, const BatchArgs bat) {
   using Tl = Tile<WPR, TH, H>;
   if (threadIdx.x >= kResolveThreads) {
     if (!BATCH && a0.draws_out)
@@ -1371,6 +1439,28 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
     if (tid == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&s_roots_bar)) : "memory");
   }
 
+  if (LABELS) {
+    // ---- canonical labels, a site per thread and step so that a warp writes
+    // 128 consecutive bytes: bound by the 4 B a site of its output. (A run
+    // per thread, its sites written one by one, spread every store over 32
+    // rows: L = 8192 in 735 us a call, 419 us so.)
+#pragma unroll 4
+    for (int i = tid; i < P.nrows * TW; i += NT) {
+      const int y = i / TW, x = i % TW;
+      if (x >= P.ncols) continue;
+      const int rt = par[par[i]];  // the site's label, then the label's root
+      int key;
+      if ((s_bmask[rt >> 5] >> (rt & 31)) & 1u) {
+        const int sl = slot_of(s_bmask, s_pre, rt);
+        key = sl < nsl ? s_slotkey[sl] : 0;
+      } else {
+        key = (int)((uint32_t)(P.y0 + rt / TW) * (uint32_t)L + (uint32_t)(P.x0 + rt % TW));
+      }
+      a.labels[(size_t)(P.y0 + y) * L + P.x0 + x] = key;
+    }
+    return true;
+  }
+
   // ---- per run: its root's decision; new spins of my strip. A row of labels
   // is 256 bytes, so the rows all start in bank 0, and every row word has a
   // run start at its column 0: walked in column order, the 32 lanes' first
@@ -1380,6 +1470,9 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
   // run's decision at its start, and spread the decisions over the runs
   // afterwards with a segmented prefix OR.
   const int rot = ((k & 7) << 2) | ((w >> 1 & 1) << 1);
+  // rows of whole 16-byte aligned words are stored by the threads that own
+  // them, others by the block together once all words are known
+  const bool vecrows = g.aligned16 && (P.ncols & 31) == 0;
   // HIST: a lane adds up the lengths of consecutive runs of one root and
   // sends the sum when the root changes (a tile's runs mostly belong to few
   // clusters near order, which made per-run shared atomics serialise)
@@ -1392,24 +1485,7 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
     if (r >= nv || !wmask) continue;
     const int y = y0r + r, base = y * TW + 32 * w;
     const uint32_t Rall = ~(e_int[r] << 1) & wmask;  // run starts
-    if (LABELS) {
-      uint32_t R = Rall;
-      while (R) {
-        const int b = __ffs(R) - 1;
-        R &= R - 1;
-        const int rt = par[par[base + b]];  // the run's label, then the label's root
-        const int nxt = R ? (__ffs(R) - 1) : nb;
-        int key;
-        if ((s_bmask[rt >> 5] >> (rt & 31)) & 1u) {
-          const int sl = slot_of(s_bmask, s_pre, rt);
-          key = sl < nsl ? s_slotkey[sl] : 0;
-        } else {
-          key = (int)((uint32_t)(P.y0 + rt / TW) * (uint32_t)L + (uint32_t)(P.x0 + rt % TW));
-        }
-        int32_t* out = a.labels + (size_t)(P.y0 + y) * L + P.x0 + 32 * w;
-        for (int x = b; x < nxt; ++x) out[x] = key;
-      }
-    } else {
+    {
       uint32_t Rr = __funnelshift_r(Rall, Rall, rot);  // bit i: run start at column (i + rot) mod 32
       uint32_t D = 0u;                                // decision of each run, at its start
       while (Rr) {
@@ -1441,10 +1517,9 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
       G &= G << 8;
       D |= (D << 16) & G;
       snew[r] = (a.rule ? 0u : s[r]) ^ (D & wmask);
-      store_spin_bits(a.spins_out + (size_t)(P.y0 + y) * L + P.x0 + 32 * w, snew[r], nb, g.aligned16);
+      if (vecrows) store_spin_bits(a.spins_out + (size_t)(P.y0 + y) * L + P.x0 + 32 * w, snew[r]);
     }
   }
-  if (LABELS) return true;
   if (HIST) {  // the lanes' last sums: one atomic per root and warp
     __syncwarp();
     const uint32_t peers = __match_any_sync(0xffffffffu, acc_rt);
@@ -1455,6 +1530,13 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
   for (int r = 0; r < H; ++r) s_snew[y0r + r][w] = snew[r];
 
   __syncthreads();
+
+  if (!vecrows)  // bits x .. x + 3 of the row's words (x = -3 .. -1: bit 0 on, shifted up)
+    store_rows4<TW, NT>(a.spins_out + (size_t)P.y0 * L + P.x0, L, P.nrows, P.ncols, [&](int y, int x) {
+      if (x < 0) return spin_bytes4((s_snew[y][0] << -x) & 0xFu);
+      const int ww = x >> 5;
+      return spin_bytes4(__funnelshift_r(s_snew[y][ww], ww + 1 < WPR ? s_snew[y][ww + 1] : 0u, x & 31) & 0xFu);
+    });
 
   // ---- E and M of the new state (C10)
   int eloc = 0, mloc = 0;
@@ -1752,11 +1834,11 @@ cudaError_t launch_fused_shape(const BatchArgs& b, int ntiles, int nsweeps, cuda
 
 // Phase 1 of a q-state Potts sweep: the Ising phase 1 with the bond masks of
 // equal states (phase1_body's POTTS form).
-template <int WPR, int TH, int H>
+template <int WPR, int TH, int H, bool ALIGNED>
 __global__ void __launch_bounds__(32 * WPR, band_min_blocks<32 * WPR>())
     potts_phase1_kernel(const SweepArgs a) {
   __shared__ P1Shared<WPR, TH, H> S;
-  phase1_body<WPR, TH, H, false, false, true>(S, a, BatchArgs{}, blockIdx.x, 0);
+  phase1_body<WPR, TH, H, false, false, true, ALIGNED>(S, a, BatchArgs{}, blockIdx.x, 0);
 }
 
 constexpr int kPottsP3Threads = 256;  // threads per tile of the Potts phase 3
@@ -1781,7 +1863,8 @@ struct PottsP3Shared {
 // an inner one drawn here from its root's key), every site its cluster's, and
 // E = -(edges joining equal states), M = (sites in state 0) of the new
 // configuration are summed in int64.
-template <int WPR, int TH, int H>
+// ALIGNED: L is a multiple of 16 (every four sites are one aligned store).
+template <int WPR, int TH, int H, bool ALIGNED>
 __global__ void __launch_bounds__(kPottsP3Threads) potts_phase3_kernel(const SweepArgs a) {
   using Tl = Tile<WPR, TH, H>;
   constexpr int TW = Tl::TW, NT = kPottsP3Threads, NB = Tl::NB, MS = Tl::MS, RW = Tl::RW;
@@ -1875,14 +1958,16 @@ __global__ void __launch_bounds__(kPottsP3Threads) potts_phase3_kernel(const Swe
     for (int k = 0; k < 4; ++k)
       if (x + k < P.ncols) word |= (uint32_t)S.val[S.par[S.par[base + k]]] << (8 * k);
     *reinterpret_cast<uint32_t*>(&S.snew[y][x]) = word;
-    int8_t* out = a.spins_out + (size_t)(P.y0 + y) * L + P.x0 + x;
-    if (g.aligned16 && x + 4 <= P.ncols) {
-      *reinterpret_cast<uint32_t*>(out) = word;
-    } else {
-      for (int k = 0; k < 4 && x + k < P.ncols; ++k) out[k] = (int8_t)(word >> (8 * k));
-    }
+    if (ALIGNED) *reinterpret_cast<uint32_t*>(a.spins_out + (size_t)(P.y0 + y) * L + P.x0 + x) = word;
   }
   __syncthreads();
+  if (!ALIGNED)
+    store_rows4<TW, NT>(a.spins_out + (size_t)P.y0 * L + P.x0, L, P.nrows, P.ncols, [&](int y, int x) {
+      const uint32_t* row = reinterpret_cast<const uint32_t*>(&S.snew[y][0]);
+      if (x < 0) return row[0] << (-8 * x);
+      const int q = x >> 2;
+      return __funnelshift_r(row[q], q + 1 < G ? row[q + 1] : 0u, 8 * (x & 3));
+    });
 
   // ---- E and M of the new states: east and south edge of every site
   long long e = 0, m = 0;
@@ -2082,13 +2167,17 @@ cudaError_t launch_export_bonds(int shape, const SweepArgs& a, uint8_t* out, cud
 
 cudaError_t launch_potts_phase1(const SweepArgs& a, cudaStream_t st) {
   constexpr TileShape ts = shape_of(kPottsShape);
-  potts_phase1_kernel<ts.wpr, ts.th, ts.h><<<a.g.tiles_x * a.g.tiles_y, 32 * ts.wpr, 0, st>>>(a);
+  const int n = a.g.tiles_x * a.g.tiles_y;
+  if (a.g.aligned16) potts_phase1_kernel<ts.wpr, ts.th, ts.h, true><<<n, 32 * ts.wpr, 0, st>>>(a);
+  else potts_phase1_kernel<ts.wpr, ts.th, ts.h, false><<<n, 32 * ts.wpr, 0, st>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_potts_phase3(const SweepArgs& a, cudaStream_t st) {
   constexpr TileShape ts = shape_of(kPottsShape);
-  potts_phase3_kernel<ts.wpr, ts.th, ts.h><<<a.g.tiles_x * a.g.tiles_y, kPottsP3Threads, 0, st>>>(a);
+  const int n = a.g.tiles_x * a.g.tiles_y;
+  if (a.g.aligned16) potts_phase3_kernel<ts.wpr, ts.th, ts.h, true><<<n, kPottsP3Threads, 0, st>>>(a);
+  else potts_phase3_kernel<ts.wpr, ts.th, ts.h, false><<<n, kPottsP3Threads, 0, st>>>(a);
   return cudaGetLastError();
 }
 

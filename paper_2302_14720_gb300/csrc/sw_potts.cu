@@ -201,7 +201,7 @@ int sw_potts_create(int32_t L, int32_t q, double beta, uint64_t seed, int32_t in
     e = cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking);
     h->own_stream = e == cudaSuccess;
   }
-  if (e == cudaSuccess) e = cudaMalloc(&h->s, n);
+  if (e == cudaSuccess) e = cudaMalloc(&h->s, n + sw::kPottsPad);
   if (e == cudaSuccess) e = cudaMalloc(&h->tb.tbits, ntiles * 3 * ts.row_words() * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&h->tb.roots, ntiles * ts.sites() * sizeof(uint16_t));
   if (e == cudaSuccess) e = cudaMalloc(&h->tb.bmask, ntiles * ts.row_words() * sizeof(uint32_t));
