@@ -160,9 +160,16 @@ cudaError_t launch_batch_fused(int shape, const BatchArgs& b, int ntiles, int ns
 // Whole sweeps of one small lattice in one CTA (sw_small.cu). 181^2 < 2^15,
 // so 16-bit parents index every site.
 constexpr int kSmallMaxL = 181;
-// sw_sweep takes the one-CTA path up to this side; from about L = 160 on the
-// tiled path is as fast on GB300 (62 us per sweep either way at L = 160).
-constexpr int kSmallSweepMaxL = 144;
+// sw_sweep takes the one-CTA path (any L <= 256 fits) up to kSmallSweepMaxL,
+// and up to kSmallChainMaxL in calls of four sweeps or more: a sweep costs the
+// CTA less than the tiled path's launches up to about L = 220, its first one
+// twice that. Us per sweep of a 100-sweep call (with one union-find over all
+// runs, before the segments): L = 64 9.0 (15.2), 100 14.5 (37.7), 144 20.7
+// (67.0); one CTA / tiled: 181 33 / 49, 208 39 / 46, 256 57 / 46. One-sweep
+// calls with their read-back: L = 160 80 / 84, 181 97 / 84.
+constexpr int kSmallSweepMaxL = 160;
+constexpr int kSmallChainMaxL = 208;
+inline bool small_sweep(int L, int n) { return L <= kSmallSweepMaxL || (L <= kSmallChainMaxL && n >= 4); }
 struct SmallArgs {
   int L;
   uint32_t thr;    // C3

@@ -1,25 +1,43 @@
-// sw_small.cu -- whole sweeps of a small lattice (L <= kSmallMaxL) in one CTA.
+// sw_small.cu -- whole sweeps of a small lattice in one CTA.
 //
-// A lattice of at most 181 x 181 sites fits one CTA's shared memory whole:
-// spins and bonds as bit masks, and a 16-bit union-find parent per site.
-// One launch runs n sweeps back to back with block barriers between the
-// steps, so a small lattice costs no cross-tile merge and no launch per
-// phase. The steps and their results are those of the tiled path:
-//   bonds (§2.1, C5)  a warp per row word, a lane per site, the word's bond
-//                     masks assembled by ballot;
-//   clusters (§2.3)   union-find over runs (stretches of a row word joined
-//                     by east bonds), a lane per bond that joins two runs;
-//                     the larger root is hung under the smaller, so every
-//                     root is its cluster's smallest site (C9);
-//   new spins (§2.4)  the flip bits of all site indices are filled from
-//                     their blocks and each root reads its own (C6), or
-//                     each root draws C6b's fresh spin; a warp per row
-//                     word sets its 32 sites from their runs' roots;
-//   E and M (C10)     from the new bit masks, int64, one trace row per sweep.
+// A lattice of at most 256 x 256 sites fits one CTA's shared memory whole:
+// spins and bonds as bit masks, and a 16-bit label per site. One launch runs
+// n sweeps back to back with block barriers between the steps, so a small
+// lattice costs no cross-tile merge and no launch per phase. The steps and
+// their results are those of the tiled path:
+//   draws (C5)        a Philox block per pair of consecutive site indices,
+//                     straight through the lattice (pairs straddle rows of
+//                     an odd side), into flat bit strings;
+//   bonds (§2.1)      a thread per row word, which shifts its draws out of
+//                     the strings; E and M (C10) of the state fall out of the
+//                     same words, so they are summed here, one sweep late;
+//   clusters (§2.3)   a warp per segment (a 32-column band of a few rows): a
+//                     Hoshen-Kopelman scan down the segment (row_masks)
+//                     labels its runs, a warp-private union-find joins the
+//                     runs that meet, and the bonds out of the segment (east,
+//                     south, the periodic wraps) are united across warps by
+//                     compare-and-swap; the larger root is hung under the
+//                     smaller, so every root is its cluster's smallest site;
+//   new spins (§2.4)  a lane per site walks its label to the root, four rows
+//                     at a time, and takes the root's flip bit (C6; the bits
+//                     of all site indices are filled from their blocks) or
+//                     the fresh spin drawn for it (C6b).
 // Spins are read at the start and written back after the last sweep.
+//
+// What bounds it: one SM. Up to about L = 64 a sweep is a chain of four
+// barriers with dependent shared-memory loads between them, so the work is
+// cut into 32 segments (one a warp) rather than into few tall ones; above,
+// the instructions of the Philox blocks and of the scan. Cycles of a sweep at
+// L = 64 (18.6 k): draws 2.4 k, bonds 0.6 k, scan 2.0 k, unions inside a
+// segment 3.0 k, across segments 4.6 k, walks and new spins 5.4 k. Measured
+// and not kept: half the warps drawing the next sweep's blocks while the
+// others label (9.3 us against 9.0 at L = 64, 27 against 21 at 144), and
+// pointing every label at its root before the sites look (10.9 from work
+// lists, 9.7 in step).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "sw_band.cuh"
 #include "sw_internal.h"
 #include "sw_philox.cuh"
 
@@ -28,71 +46,86 @@ namespace {
 
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallUnionCap = 1 << 20;
+constexpr int kSmallMinRows = 4;    // rows of a segment at least
+constexpr int kSmallListCap = 128;  // entries of a warp's work list
 
-// Hang root a under b if a is still a root: one 16-bit compare-and-swap of
-// par[a] from a to b. Returns the entry found (a on success).
-__device__ __forceinline__ int small_link_root(uint16_t* par, int a, int b) {
-  return (int)atomicCAS(reinterpret_cast<unsigned short*>(par + a), (unsigned short)a, (unsigned short)b);
-}
-
-// Root of x while other threads may be uniting (path halving).
-__device__ __forceinline__ int small_find(volatile uint16_t* par, int x) {
-  for (;;) {
-    const int p = par[x];
-    if (p == x) return x;
-    const int gp = par[p];
-    if (gp == p) return p;
-    par[x] = (uint16_t)gp;
-    x = gp;
-  }
-}
-
-__device__ void small_unite(uint16_t* par, int a, int b, int* err) {
-  for (int it = 0; it < kSmallUnionCap; ++it) {
-    a = small_find(par, a);
-    b = small_find(par, b);
-    if (a == b) return;
-    if (a < b) {
-      const int tmp = a;
-      a = b;
-      b = tmp;
+// Sizes of a lattice's pieces in shared memory.
+struct SmallShape {
+  int N, WPL, RWN, DW;   // sites, words a row, row words, flat words
+  int S, nseg;           // rows of a segment, segments
+  __host__ __device__ explicit SmallShape(int L) {
+    N = L * L;
+    WPL = (L + 31) >> 5;
+    RWN = L * WPL;
+    DW = (N + 31) >> 5;
+    // as many segments a warp as keep a segment within 32 rows (a lane holds
+    // a row's masks), the rows spread evenly over them
+    for (int per_warp = 1;; ++per_warp) {
+      const int bands = per_warp * (kSmallThreads / 32) / WPL;
+      S = (L + bands - 1) / bands;
+      if (S <= 32) break;
     }
-    const int old = small_link_root(par, a, b);
-    if (old == a) return;
-    a = old;  // another thread linked a first: carry on from its new parent
+    if (S < kSmallMinRows) S = kSmallMinRows;
+    nseg = WPL * ((L + S - 1) / S);
   }
-  atomicCAS(err, 0, 1);
-}
+};
 
-// Highest run start at or below bit b of a word (R always has bit 0 set).
-__device__ __forceinline__ int small_run_start(uint32_t R, int b) {
-  return 31 - __clz(R & (0xffffffffu >> (31 - b)));
-}
-
-template <typename T>
-__device__ __forceinline__ T small_warp_sum(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+// The draws of sweep t by the whole block: the C5 bits by site index into rawE / rawS, lane p taking the block of sites 2p and 2p + 1
+// (four lanes' bits make a byte of each string), and under the flip rule the
+// C6 bits of all site indices into dec (word k of it is word k & 3 of block
+// k >> 2).
+__device__ __forceinline__ void small_draws(const SmallArgs& a, int N, int DW, uint32_t t, uint32_t* rawE,
+                                            uint32_t* rawS, uint32_t* dec) {
+  constexpr int nw = kSmallThreads / 32;
+  const int lane = threadIdx.x & 31, i = threadIdx.x >> 5;
+  const int np = (((N + 1) >> 1) + 3) & ~3;
+  uint8_t* rawE8 = reinterpret_cast<uint8_t*>(rawE);
+  uint8_t* rawS8 = reinterpret_cast<uint8_t*>(rawS);
+  for (int p0 = 32 * i; p0 < np; p0 += 32 * nw) {
+    const int p = p0 + lane, sh = 2 * (p & 3);
+    const uint4 q = philox4x32_10(make_uint4((uint32_t)p, t, 0u, 0u), a.ks);
+    uint32_t v = (((uint32_t)(q.x < a.thr) | ((uint32_t)(q.z < a.thr) << 1)) << sh) |
+                 (((uint32_t)(q.y < a.thr) | ((uint32_t)(q.w < a.thr) << 1)) << (8 + sh));
+    v |= __shfl_xor_sync(0xffffffffu, v, 1);
+    v |= __shfl_xor_sync(0xffffffffu, v, 2);
+    if ((lane & 3) == 0 && p < np) {
+      rawE8[p >> 2] = (uint8_t)v;
+      rawS8[p >> 2] = (uint8_t)(v >> 8);
+    }
+  }
+  if (a.rule == 0) {
+    for (int b = 32 * (nw - 1 - i) + lane; 4 * b < DW; b += 32 * nw) {
+      const uint4 q = philox4x32_10(make_uint4((uint32_t)b, t, 1u, 0u), a.ks);
+      dec[4 * b] = q.x;
+      if (4 * b + 1 < DW) dec[4 * b + 1] = q.y;
+      if (4 * b + 2 < DW) dec[4 * b + 2] = q.z;
+      if (4 * b + 3 < DW) dec[4 * b + 3] = q.w;
+    }
+  }
 }
 
 // The n sweeps of one lattice by the whole CTA (smem: small_smem_bytes(L)).
 __device__ __forceinline__ void small_body(const SmallArgs& a, uint32_t* smem) {
   constexpr int NT = kSmallThreads, NW = NT / 32;
-  __shared__ long long s_red[2][NW];
-  __shared__ uint16_t s_rootq[NW][64];  // roots waiting for their draw
-  const int L = a.L, N = L * L, WPL = (L + 31) >> 5, RWN = L * WPL, DW = (N + 31) >> 5;
-  uint32_t* s_spin = smem;       // [RWN] sign bits (1 = -1)
-  uint32_t* s_e = s_spin + RWN;  // [RWN] east bonds
-  uint32_t* s_s = s_e + RWN;     // [RWN] south bonds
-  uint32_t* s_dec = s_s + RWN;   // [DW] decision bit of every root
-  uint16_t* par = reinterpret_cast<uint16_t*>(s_dec + DW);  // [N]
+  __shared__ uint16_t s_list[NW][kSmallListCap];  // a warp's unions, its labels, roots waiting for their draw
+  __shared__ int s_em[2];
+  const SmallShape Z(a.L);
+  const int L = a.L, N = Z.N, WPL = Z.WPL, RWN = Z.RWN, DW = Z.DW;
+  uint32_t* s_spin = smem;        // [RWN] sign bits (1 = -1)
+  uint32_t* s_e = s_spin + RWN;   // [RWN] east bonds
+  uint32_t* s_s = s_e + RWN;      // [RWN] south bonds
+  uint32_t* s_new = s_s + RWN;    // [RWN] sites that name a label of their own
+  uint32_t* s_dec = s_new + RWN;  // [2][DW] decision bit of every root, by sweep parity
+  uint32_t* rawE = s_dec + 2 * DW;   // [DW + 1] draws by site index, east
+  uint32_t* rawS = rawE + DW + 1;    // [DW + 1] south
+  uint16_t* par = reinterpret_cast<uint16_t*>(rawS + DW + 1);  // [N] labels; a label's entry is its parent
+  volatile uint16_t* vpar = par;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // lanes per row word for bonds and unions: as many as the threads allow
-  // (a power of two, at most 32), each taking 32 / G consecutive columns
-  int G = 1;
-  while (G < 32 && 2 * G * RWN <= NT) G *= 2;
-  const int PER = 32 / G, sub = lane % G;
+  const bool flip_rule = a.rule == 0;
+  // this thread's first row word, and the step to its next
+  const int ry0 = tid / WPL, rw0 = tid - ry0 * WPL, rdy = NT / WPL, rdw = NT - rdy * WPL;
+  // this warp's first segment (band sw0, rows from sj0 * S on), and the step to its next
+  const int sj0 = warp / WPL, sw0 = warp - sj0 * WPL, sdj = NW / WPL, sdw = NW - sdj * WPL;
 
   for (int rw = warp; rw < RWN; rw += NW) {
     const int y = rw / WPL, x = (rw % WPL) * 32 + lane;
@@ -100,187 +133,288 @@ __device__ __forceinline__ void small_body(const SmallArgs& a, uint32_t* smem) {
     const uint32_t m = __ballot_sync(0xffffffffu, minus);
     if (lane == 0) s_spin[rw] = m;
   }
-  __syncthreads();
-
-  for (int k = 0; k < a.n; ++k) {
+  if (tid < 2) s_em[tid] = 0;
+  for (int k = 0;; ++k) {
     const uint32_t t = a.t0 + (uint32_t)k;
-    for (int i = tid; i < DW; i += NT) s_dec[i] = 0u;
-    for (int i = tid; i < N; i += NT) par[i] = (uint16_t)i;
+    uint32_t* dec = s_dec + (k & 1) * DW;  // (the sweep before's may still be read)
+    if (k < a.n) small_draws(a, N, DW, t, rawE, rawS, dec);
+    __syncthreads();
 
-    // ---- bonds (§2.1): G lanes per row word, each drawing a stretch of
-    // 32 / G sites (one block for the two sites of a pair when both lie in
-    // its stretch, C5); the word's masks are or-reduced across the G lanes
-    for (int rw0 = warp * (32 / G); rw0 < RWN; rw0 += NT / G) {
-      const int rw = rw0 + lane / G;
-      uint32_t eb = 0u, sb = 0u;
-      int y = 0, w = 0, nb = 0;
+    // ---- E and M (C10) of the state, that of the sweep before, and the bonds
+    // (§2.1) of this sweep
+    for (int rw = tid, y = ry0, w = rw0, r0 = tid & ~31; r0 < RWN; r0 += NT, rw += NT) {
+      int e = 0, m = 0;
       if (rw < RWN) {
-        y = rw / WPL;
-        w = rw % WPL;
-        nb = min(32, L - 32 * w);
-        const uint32_t i0 = (uint32_t)(y * L + 32 * w);
-        const int b1 = min(nb, sub * PER + PER);
-        for (int b = sub * PER; b < b1; ++b) {
-          const uint32_t i = i0 + b;
-          const uint4 q = philox4x32_10(make_uint4(i >> 1, t, 0u, 0u), a.ks);
-          if ((i & 1u) == 0u && b + 1 < b1) {  // both sites of the pair
-            eb |= ((uint32_t)(q.x < a.thr) << b) | ((uint32_t)(q.z < a.thr) << (b + 1));
-            sb |= ((uint32_t)(q.y < a.thr) << b) | ((uint32_t)(q.w < a.thr) << (b + 1));
-            ++b;
-          } else {
-            eb |= (uint32_t)(((i & 1u) ? q.z : q.x) < a.thr) << b;
-            sb |= (uint32_t)(((i & 1u) ? q.w : q.y) < a.thr) << b;
-          }
-        }
-      }
-      for (int o = 1; o < G; o <<= 1) {
-        eb |= __shfl_xor_sync(0xffffffffu, eb, o);
-        sb |= __shfl_xor_sync(0xffffffffu, sb, o);
-      }
-      if (rw < RWN && sub == 0) {
-        const uint32_t vm = nb == 32 ? 0xffffffffu : ((1u << nb) - 1u);
+        const int nb = min(32, L - 32 * w);
+        const uint32_t vm = 0xffffffffu >> (32 - nb);
         const uint32_t sp = s_spin[rw];
         // east neighbours: the next site in the word; the word's last site
         // meets the next word's first, or column 0 of its row (periodic)
-        const uint32_t nxt = w + 1 < WPL ? s_spin[rw + 1] : s_spin[y * WPL];
-        const uint32_t sE = ((sp >> 1) & (vm >> 1)) | ((nxt & 1u) << (nb - 1));
-        const uint32_t sS = s_spin[(y + 1 == L ? 0 : y + 1) * WPL + w];
-        s_e[rw] = eb & ~(sp ^ sE) & vm;
-        s_s[rw] = sb & ~(sp ^ sS) & vm;
+        const uint32_t nxt = s_spin[w + 1 < WPL ? rw + 1 : y * WPL];
+        const uint32_t dE = (sp ^ (((sp >> 1) & (vm >> 1)) | ((nxt & 1u) << (nb - 1)))) & vm;
+        const uint32_t dS = (sp ^ s_spin[y + 1 == L ? w : rw + WPL]) & vm;
+        e = 2 * (__popc(dE) + __popc(dS)) - 2 * nb;
+        m = nb - 2 * __popc(sp & vm);
+        const int i0 = y * L + 32 * w, q = i0 >> 5, o = i0 & 31;
+        s_e[rw] = __funnelshift_r(rawE[q], rawE[q + 1], o) & ~dE & vm;
+        s_s[rw] = __funnelshift_r(rawS[q], rawS[q + 1], o) & ~dS & vm;
+      }
+      e = __reduce_add_sync(0xffffffffu, e);
+      m = __reduce_add_sync(0xffffffffu, m);
+      if (lane == 0) {
+        atomicAdd(&s_em[0], e);
+        atomicAdd(&s_em[1], m);
+      }
+      y += rdy;
+      w += rdw;
+      if (w >= WPL) {
+        w -= WPL;
+        ++y;
       }
     }
+    if (!flip_rule)
+      for (int i = tid; i < DW; i += NT) dec[i] = 0u;
     __syncthreads();
-
-    // ---- clusters (§2.3) over runs: a run is a stretch of a row word
-    // joined by east bonds inside the word, and its first site is its
-    // union-find node. Unions join the runs that the bonds between words,
-    // across the row's periodic wrap and between rows connect; the larger
-    // node is hung under the smaller, so every root is its cluster's
-    // smallest site (C9: a cluster's smallest site starts a run). G lanes
-    // share a row word, each uniting the bonds of its 32 / G columns in turn.
-    for (int rw = tid / G; rw < RWN; rw += NT / G) {
-      const int y = rw / WPL, w = rw % WPL, nb = min(32, L - 32 * w);
-      const uint32_t vm = nb == 32 ? 0xffffffffu : ((1u << nb) - 1u), lastb = 1u << (nb - 1);
-      const uint32_t mine = (PER == 32 ? 0xffffffffu : ((1u << PER) - 1u)) << (sub * PER);
-      const uint32_t e = s_e[rw], ein = e & ~lastb, R = ~(ein << 1) & vm;
-      const int base = y * L + 32 * w;
-      const int yn = y + 1 == L ? 0 : y + 1, rwn = yn * WPL + w, basen = yn * L + 32 * w;
-      const uint32_t en = s_e[rwn] & ~lastb, Rn = ~(en << 1) & vm, d = s_s[rw];
-      // a south bond is redundant when the one left of it joins the same two runs
-      uint32_t need = d & ~((d & ein & en) << 1) & mine;
-      while (need) {
-        const int j = __ffs(need) - 1;
-        need &= need - 1;
-        small_unite(par, base + small_run_start(R, j), basen + small_run_start(Rn, j), a.err);
-      }
-      if ((e & lastb & mine) != 0u)
-        small_unite(par, base + small_run_start(R, nb - 1), w + 1 < WPL ? base + nb : y * L, a.err);
+    if (tid < 2) {
+      if (k > 0) a.em[2 * (k - 1) + tid] = s_em[tid];
+      s_em[tid] = 0;
     }
-    __syncthreads();
+    if (k == a.n) break;
 
-    // ---- every run start points at its root; roots draw their decision. Flip
-    // rule (C6): word k of s_dec, the bits of site indices 32k .. 32k+31, is
-    // word k & 3 of block k >> 2, so every word is filled from its block and
-    // each root reads its own bit. Assignment rule (C6b): the roots are
-    // queued per warp and drawn 32 at a time so that every lane draws.
-    const bool flip_rule = a.rule == 0;
-    if (flip_rule) {
-      for (int b = tid; 4 * b < DW; b += NT) {
-        const uint4 q4 = philox4x32_10(make_uint4((uint32_t)b, t, 1u, 0u), a.ks);
-        s_dec[4 * b] = q4.x;
-        if (4 * b + 1 < DW) s_dec[4 * b + 1] = q4.y;
-        if (4 * b + 2 < DW) s_dec[4 * b + 2] = q4.z;
-        if (4 * b + 3 < DW) s_dec[4 * b + 3] = q4.w;
+    // ---- clusters (§2.3) inside each segment: lane l holds the masks of
+    // the segment's row l; the warp scans the rows top to bottom, lane l
+    // holding column l (see phase 1 of the tiled path)
+    uint16_t* list = s_list[warp];
+    for (int seg = warp, j = sj0, w = sw0; seg < Z.nseg; seg += NW) {
+      const int y0 = j * Z.S, n = min(Z.S, L - y0), nb = min(32, L - 32 * w);
+      const int org = y0 * L + 32 * w;  // the segment's first site
+      const uint32_t vm = 0xffffffffu >> (32 - nb);
+      RowMasks m{0u, 0u, 0u, 0u};
+      if (lane < n) {
+        const int rw = (y0 + lane) * WPL + w;
+        const bool up = lane > 0;
+        m = row_masks(s_e[rw] & (vm >> 1), vm, up ? s_e[rw - WPL] & (vm >> 1) : 0u, up ? vm : 0u,
+                      up ? s_s[rw - WPL] : 0u);
+        s_new[rw] = m.S & ~m.F;
       }
-    }
-    {
-      uint16_t* q = s_rootq[warp];
-      int qh = 0, qn = 0;  // the same in every lane of the warp
-      for (int i0 = warp * 32; i0 < N; i0 += NT) {
-        const int i = i0 + lane;
-        bool isroot = false;
-        if (i < N) {
-          const int y = i / L, x = i - y * L;
-          const bool starts = (x & 31) == 0 || !((s_e[y * WPL + (x >> 5)] >> ((x & 31) - 1)) & 1u);
-          if (starts) {
-            int r = i, p = par[r];
-            while (p != r) {
-              r = p;
-              p = par[r];
+      {
+        const uint32_t le = 0xffffffffu >> (31 - lane);
+        uint32_t lab = 0u;
+        int own = org + lane;
+#pragma unroll 4
+        for (int r = 0; r < n; ++r) {
+          const uint32_t R = __shfl_sync(0xffffffffu, m.R, r);
+          const uint32_t S = __shfl_sync(0xffffffffu, m.S, r);
+          const uint32_t F = __shfl_sync(0xffffffffu, m.F, r);
+          const int s = 31 - __clz(R & le);
+          const int src = __ffs(S & (0xffffffffu << s)) - 1;
+          const uint32_t v = ((F >> lane) & 1u) ? lab : (uint32_t)own;
+          lab = __shfl_sync(0xffffffffu, v, src & 31);
+          if (lane < nb) par[own] = (uint16_t)lab;
+          own += L;
+        }
+      }
+      __syncwarp();
+      // the unions M asks for, from a list, one state machine a lane. Only
+      // this warp touches the segment's labels, so a link is a plain store
+      // checked after __syncwarp.
+      const int cnt = __popc(m.M), first = warp_exclusive_sum(cnt, lane);
+      const int total = __shfl_sync(0xffffffffu, first + cnt, 31);
+      for (int r0 = 0; r0 < total; r0 += kSmallListCap) {
+        int idx = first;
+        for (uint32_t mm = m.M; mm; mm &= mm - 1, ++idx)
+          if (idx >= r0 && idx < r0 + kSmallListCap) list[idx - r0] = (uint16_t)(org + lane * L + __ffs(mm) - 1);
+        __syncwarp();
+        const int nu = min(kSmallListCap, total - r0);
+        int q = lane, xa = 0, xb = 0;
+        bool busy = false;
+        for (int it = 0;; ++it) {
+          if (!busy && q < nu) {
+            xb = list[q];
+            xa = xb - L;
+            q += 32;
+            busy = true;
+          }
+          if (!__any_sync(0xffffffffu, busy)) break;
+          if (it >= kSmallUnionCap) {
+            if (busy) atomicCAS(a.err, 0, kErrUnionCap);
+            break;
+          }
+          int hi = -1, lo = 0;
+          if (busy) {
+            const int pa = vpar[xa], pb = vpar[xb];
+            if (pa == xa && pb == xb) {
+              if (xa == xb) {
+                busy = false;
+              } else {
+                hi = max(xa, xb);
+                lo = min(xa, xb);
+                vpar[hi] = (uint16_t)lo;
+              }
+            } else {
+              const int ga = vpar[pa], gb = vpar[pb];
+              if (ga != pa) vpar[xa] = (uint16_t)ga;
+              if (gb != pb) vpar[xb] = (uint16_t)gb;
+              xa = ga;
+              xb = gb;
             }
-            par[i] = (uint16_t)r;  // concurrent stores all write roots
-            isroot = r == i && !flip_rule;
+          }
+          __syncwarp();
+          if (hi >= 0) {
+            const int now = vpar[hi];
+            busy = now != lo;
+            xa = now;
+            xb = lo;
           }
         }
-        const uint32_t m = __ballot_sync(0xffffffffu, isroot);
-        if (isroot) q[(qh + qn + __popc(m & ((1u << lane) - 1u))) & 63] = (uint16_t)i;
-        qn += __popc(m);
+        __syncwarp();
+      }
+      j += sdj;
+      w += sdw;
+      if (w >= WPL) {
+        w -= WPL;
+        ++j;
+      }
+    }
+    __syncthreads();
+
+    // ---- the bonds out of each segment, united by compare-and-swap: lane l
+    // has the south bond of column l of its last row (unless the one left of
+    // it joins the same two runs), then the east bond out of its row l
+    // (unless the row above has one and both ends hang on it). The lanes
+    // walk to their roots first, and lanes with the same pair of roots leave
+    // it to the lowest of them: most bonds join the same few clusters.
+    for (int seg = warp, j = sj0, w = sw0; seg < Z.nseg; seg += NW) {
+      const int y0 = j * Z.S, n = min(Z.S, L - y0), nb = min(32, L - 32 * w);
+      const uint32_t vm = 0xffffffffu >> (32 - nb), lastb = 1u << (nb - 1);
+      const int yl = y0 + n - 1, yn = yl + 1 == L ? 0 : yl + 1, wn = w + 1 < WPL ? w + 1 : 0;
+      const uint32_t d = s_s[yl * WPL + w];
+      const uint32_t need = d & ~((d & s_e[yl * WPL + w] & s_e[yn * WPL + w] & (vm >> 1)) << 1);
+      bool east = false;
+      if (lane < n) {
+        const int rw = (y0 + lane) * WPL + w, rn = (y0 + lane) * WPL + wn;
+        east = (s_e[rw] & lastb) != 0u;
+        if (lane > 0 && (s_e[rw - WPL] & s_s[rw - WPL] & lastb) && (s_s[rn - WPL] & 1u)) east = false;
+      }
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
+        bool busy = pass == 0 ? ((need >> lane) & 1u) != 0u : east;
+        int xa = 0, xb = 0;
+        if (busy) {
+          xa = vpar[pass == 0 ? yl * L + 32 * w + lane : (y0 + lane) * L + 32 * w + nb - 1];
+          xb = vpar[pass == 0 ? yn * L + 32 * w + lane : (y0 + lane) * L + 32 * wn];
+        }
+        for (bool more = true; __any_sync(0xffffffffu, more);) {
+          const int pa = vpar[xa], pb = vpar[xb];
+          more = busy && (pa != xa || pb != xb);
+          xa = pa;
+          xb = pb;
+        }
+        busy = busy && xa != xb;
+        {
+          const uint32_t key = busy ? (uint32_t)(xa > xb ? xa << 16 | xb : xb << 16 | xa) : 0u;
+          const uint32_t peers = __match_any_sync(0xffffffffu, key);
+          busy = busy && lane == __ffs(peers) - 1;
+        }
+        for (int it = 0; __any_sync(0xffffffffu, busy); ++it) {
+          if (it >= kSmallUnionCap) {
+            if (busy) atomicCAS(a.err, 0, kErrUnionCap);
+            break;
+          }
+          if (busy) {
+            const int pa = vpar[xa], pb = vpar[xb];
+            if (pa == xa && pb == xb) {
+              if (xa == xb) {
+                busy = false;
+              } else {
+                const int hi = max(xa, xb), lo = min(xa, xb);
+                const int old = (int)atomicCAS(par + hi, (uint16_t)hi, (uint16_t)lo);
+                busy = old != hi;
+                xa = old;  // on failure: the root's new parent
+                xb = lo;
+              }
+            } else {
+              const int ga = vpar[pa], gb = vpar[pb];
+              if (ga != pa) vpar[xa] = (uint16_t)ga;
+              if (gb != pb) vpar[xb] = (uint16_t)gb;
+              xa = ga;
+              xb = gb;
+            }
+          }
+        }
+      }
+      j += sdj;
+      w += sdw;
+      if (w >= WPL) {
+        w -= WPL;
+        ++j;
+      }
+    }
+    __syncthreads();
+
+    // ---- assignment rule (C6b): the roots are queued per warp and drawn 32
+    // at a time so that every lane draws
+    if (!flip_rule) {
+      int qh = 0, qn = 0;  // the same in every lane of the warp
+      auto draw = [&](int x) {
+        if (decision_bit((uint32_t)x, t, a.ks, a.rule)) atomicOr(&dec[x >> 5], 1u << (x & 31));
+      };
+      for (int rw = warp; rw < RWN; rw += NW) {
+        const int y = rw / WPL, x = y * L + 32 * (rw - y * WPL) + lane;
+        const bool isroot = ((s_new[rw] >> lane) & 1u) && par[x] == x;
+        const uint32_t mr = __ballot_sync(0xffffffffu, isroot);
+        if (isroot) list[(qh + qn + __popc(mr & ((1u << lane) - 1u))) & 63] = (uint16_t)x;
+        qn += __popc(mr);
         __syncwarp();
         if (qn >= 32) {
-          const int x = q[(qh + lane) & 63];
-          if (decision_bit((uint32_t)x, t, a.ks, a.rule)) atomicOr(&s_dec[x >> 5], 1u << (x & 31));
+          draw(list[(qh + lane) & 63]);
           qh += 32;
           qn -= 32;
           __syncwarp();
         }
       }
-      if (lane < qn) {
-        const int x = q[(qh + lane) & 63];
-        if (decision_bit((uint32_t)x, t, a.ks, a.rule)) atomicOr(&s_dec[x >> 5], 1u << (x & 31));
-      }
+      if (lane < qn) draw(list[(qh + lane) & 63]);
+      __syncthreads();
     }
-    __syncthreads();
 
-    // ---- new spins (§2.4): a warp per row word, a lane per site, each site
-    // taking the decision of its run's root
-    for (int rw = warp; rw < RWN; rw += NW) {
-      const int y = rw / WPL, w = rw % WPL, nb = min(32, L - 32 * w);
-      bool d = false;
-      if (lane < nb) {
-        const uint32_t vm = nb == 32 ? 0xffffffffu : ((1u << nb) - 1u);
-        const uint32_t R = ~((s_e[rw] & ~(1u << (nb - 1))) << 1) & vm;
-        const int r = par[y * L + 32 * w + small_run_start(R, lane)];
-        d = (s_dec[r >> 5] >> (r & 31)) & 1u;
+    // ---- new spins (§2.4): every site walks from its label to the root, four
+    // rows of the warp's segment in step, and takes the root's decision
+    for (int seg = warp, j = sj0, w = sw0; seg < Z.nseg; seg += NW) {
+      const int y0 = j * Z.S, n = min(Z.S, L - y0), nb = min(32, L - 32 * w);
+      const int org = y0 * L + 32 * w + min(lane, nb - 1);
+      for (int r0 = 0; r0 < n; r0 += 4) {
+        int x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = par[org + min(r0 + i, n - 1) * L];  // past the end: the last row again
+        bool more = true;
+        while (__any_sync(0xffffffffu, more)) {
+          more = false;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int p = par[x[i]];
+            more |= p != x[i];
+            x[i] = p;
+          }
+        }
+        uint32_t mine = 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t dm = __ballot_sync(0xffffffffu, lane < nb && ((dec[x[i] >> 5] >> (x[i] & 31)) & 1u));
+          if (lane == i) mine = dm;
+        }
+        if (lane < 4 && r0 + lane < n) {  // lane i has row r0 + i
+          uint32_t* p = s_spin + (y0 + r0 + lane) * WPL + w;
+          *p = (flip_rule ? *p : 0u) ^ mine;
+        }
       }
-      const uint32_t dm = __ballot_sync(0xffffffffu, d);
-      if (lane == 0) s_spin[rw] = (a.rule ? 0u : s_spin[rw]) ^ dm;
-    }
-    __syncthreads();
-
-    // ---- E and M of the new state (C10)
-    long long e = 0, m = 0;
-    for (int rw = tid; rw < RWN; rw += NT) {
-      const int y = rw / WPL, w = rw % WPL;
-      const int nb = min(32, L - 32 * w);
-      const uint32_t vm = nb == 32 ? 0xffffffffu : ((1u << nb) - 1u);
-      const uint32_t s = s_spin[rw];
-      uint32_t sE;
-      if (32 * w + nb == L) {  // last word of the row: its last site wraps to column 0
-        sE = ((s >> 1) & (vm >> 1)) | ((s_spin[y * WPL] & 1u) << (nb - 1));
-      } else {
-        sE = (s >> 1) | ((s_spin[rw + 1] & 1u) << 31);
+      j += sdj;
+      w += sdw;
+      if (w >= WPL) {
+        w -= WPL;
+        ++j;
       }
-      const uint32_t sS = s_spin[(y + 1 == L ? 0 : y + 1) * WPL + w];
-      e += 2 * (__popc((s ^ sE) & vm) + __popc((s ^ sS) & vm)) - 2 * nb;
-      m += nb - 2 * __popc(s & vm);
     }
-    e = small_warp_sum(e);
-    m = small_warp_sum(m);
-    if (lane == 0) {
-      s_red[0][warp] = e;
-      s_red[1][warp] = m;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      long long et = 0, mt = 0;
-      for (int q = 0; q < NW; ++q) {
-        et += s_red[0][q];
-        mt += s_red[1][q];
-      }
-      a.em[2 * k] = et;
-      a.em[2 * k + 1] = mt;
-    }
-    __syncthreads();
+    // the next sweep's draws touch nothing that is still read here
   }
 
   for (int rw = warp; rw < RWN; rw += NW) {
@@ -324,16 +458,16 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
 }
 
 size_t small_smem_bytes(int L) {
-  const size_t N = (size_t)L * L, WPL = (size_t)(L + 31) / 32, RWN = (size_t)L * WPL, DW = (N + 31) / 32;
-  return (3 * RWN + DW) * sizeof(uint32_t) + N * sizeof(uint16_t);
+  const SmallShape Z(L);
+  return (4 * (size_t)Z.RWN + 4 * (size_t)Z.DW + 2) * sizeof(uint32_t) + (size_t)Z.N * sizeof(uint16_t);
 }
 
 }  // namespace
 
 cudaError_t launch_small(const SmallArgs& a, cudaStream_t st) {
-  if (a.L < 2 || a.L > kSmallMaxL) return cudaErrorInvalidValue;
+  if (a.L < 2 || a.L > kSmallChainMaxL) return cudaErrorInvalidValue;
   if (a.n <= 0) return cudaSuccess;
-  const size_t dyn = small_smem_bytes(kSmallMaxL);
+  const size_t dyn = small_smem_bytes(kSmallChainMaxL);
   static bool attr_done = false;  // set once per process; the attribute is per function
   if (!attr_done) {
     const cudaError_t e =
