@@ -142,7 +142,7 @@ def batch_candidates(shapes: Iterable[int], small=(0, 64, 181)) -> list[tuple[in
     out = []
     for sh in shapes:
         info = sw_shape_info(sh)
-        fused_ok = info["tile_h"] == 32 * info["strip_h"]
+        fused_ok = info["tile_h"] >= 64 and info["tile_h"] == 32 * info["strip_h"]
         for sched in ((SW_SCHEDULE_PHASES, SW_SCHEDULE_FUSED) if fused_ok else (SW_SCHEDULE_PHASES,)):
             for sm in small:
                 out.append((sh, sched, sm))

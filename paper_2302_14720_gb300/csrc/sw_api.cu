@@ -79,9 +79,11 @@ int shape_for(int L, bool lattice) {
   if (L <= 64) return 2;
   // A lone lattice of side <= 1024 has at most 128 tiles of 128 x 64, less
   // than one wave of 152 SMs; with 128 x 32 tiles twice as many CTAs share
-  // each phase's latency (measured on GB300 at L = 256 .. 1024: one-sweep
-  // calls 12 %, sweeps with statistics 9 % faster, chains even). Batches keep
-  // 128 x 64, whose fused schedule the 128 x 32 shape does not have.
+  // each phase's latency, and in phase 3 a thread has one row word (one-row
+  // strips) instead of two to walk. With these strips phases 1 and 3 take the
+  // same block, so that chains run them in one launch: L = 256 44.5 -> 36.7
+  // us a sweep, 1024 49.9 -> 40.3, with statistics 78 -> 64. Batches keep
+  // 128 x 64.
   return lattice && L <= 1024 ? 7 : 6;
 }
 
@@ -365,7 +367,7 @@ int sw_create(int32_t L, double beta, uint64_t seed, int32_t init, void* stream,
   if (e == cudaSuccess) e = cudaMalloc(&h->tb.err, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->csize, ntiles * ts.max_slots() * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&h->draws, ntiles * ts.row_words() * sizeof(uint2));
-  h->fuse = sw::batch_fused_supported(h->shape);
+  h->fuse = sw::phase31_supported(h->shape);
   if (e == cudaSuccess && h->fuse) e = cudaMalloc(&h->nodes2, ntiles * ts.max_slots() * sizeof(uint64_t));
   if (e == cudaSuccess && h->fuse) e = cudaMalloc(&h->bslot2, ntiles * ts.boundary_sites() * sizeof(uint16_t));
   if (e == cudaSuccess && h->fuse) e = cudaMalloc(&h->nslots2, ntiles * sizeof(int32_t));

@@ -47,7 +47,7 @@ __host__ __device__ constexpr TileShape shape_of(int v) {
          : v == 4 ? TileShape{4, 128, 4, 0}
          : v == 5 ? TileShape{8, 64, 8, 0}
          : v == 6 ? TileShape{4, 64, 2, 0}
-         : v == 7 ? TileShape{4, 32, 2, 0}
+         : v == 7 ? TileShape{4, 32, 1, 0}
          : v == 8 ? TileShape{8, 32, 2, 0}
                   : TileShape{16, 32, 2, 0};
 }
@@ -148,12 +148,14 @@ cudaError_t launch_batch_phase(int shape, int which, const BatchArgs& b, int nti
 cudaError_t launch_batch_advance(const BatchArgs& b, cudaStream_t st);
 // Batch, fused schedule: one cooperative launch runs nsweeps whole sweeps of
 // every replica with tiles (all four phases, grid barriers between them) and
-// advances the replicas' counters itself. Only shapes whose phases 1 and 3
-// take the same block (TH == 32 H) have it: batch_fused_supported.
+// advances the replicas' counters itself. Only shapes of 64 rows and more
+// whose phases 1 and 3 take the same block (TH == 32 H) have it:
+// batch_fused_supported.
 bool batch_fused_supported(int shape);
 // Phase 3 of sweep t (a3) and phase 1 of sweep t + 1 (a1) in one launch, the
 // new spins handed over in shared memory (flip or assignment rule, no
-// statistics). Same shapes as batch_fused_supported.
+// statistics). Shapes whose phases 1 and 3 take the same block.
+bool phase31_supported(int shape);
 cudaError_t launch_phase31(int shape, const SweepArgs& a3, const SweepArgs& a1, cudaStream_t st);
 cudaError_t launch_batch_fused(int shape, const BatchArgs& b, int ntiles, int nsweeps, cudaStream_t st);
 

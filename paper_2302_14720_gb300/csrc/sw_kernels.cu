@@ -556,12 +556,12 @@ __device__ __forceinline__ uint2 bond_draws(uint32_t i0, int L, uint32_t t, uint
 // Phase 1 runs one warp per 32-column band and asks for 1280 resident
 // threads an SM (at most 51 registers a thread; ten CTAs of 128 threads also
 // fit their shared memory).
-// Phase 3 runs strips of H rows; with two-row strips it asks for 1280
-// resident threads an SM as well. Taller strips would spill under that bound
+// Phase 3 runs strips of H rows; with one- and two-row strips it asks for
+// 1280 resident threads an SM as well. Taller strips would spill under that bound
 // and keep the compiler's choice.
 template <int NT, int H>
 constexpr int strip_min_blocks() {
-  return H == 2 ? 1280 / NT : 1;
+  return H <= 2 ? 1280 / NT : 1;
 }
 
 template <int NT>
@@ -1307,10 +1307,11 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
   // a row word's inner roots take their bits from one draw. Under the
   // assignment rule each root draws its own block: the lanes of a warp walk
   // their inner roots in step and queue them (in s_snew, free until the new
-  // spins); the queue is drawn 64 roots at a time, two draws per lane.
+  // spins); half the queue is drawn at a time, one or two draws per lane.
   if (!LABELS) {
     const int warp = tid >> 5;
-    constexpr int QC = 128;  // queue entries per warp
+    // queue entries per warp, as s_snew holds them; half are drawn at a time
+    constexpr int QC = 2 * TH * WPR / (NT / 32) >= 128 ? 128 : 64, QD = QC / 2;
     static_assert((NT / 32) * QC <= 2 * TH * WPR, "root queues fit in s_snew");
     uint16_t* q = reinterpret_cast<uint16_t*>(&s_snew[0][0]) + warp * QC;
     int qh = 0, qn = 0;  // the same in every lane of the warp
@@ -1349,13 +1350,19 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
         if (have) q[(qh + qn + __popc(m & ((1u << lane) - 1u))) & (QC - 1)] = (uint16_t)x;
         qn += __popc(m);
         __syncwarp();
-        if (qn >= 64) {
-          const int x0 = q[(qh + lane) & (QC - 1)], x1 = q[(qh + 32 + lane) & (QC - 1)];
-          const uint32_t f0 = draw(x0), f1 = draw(x1);
-          if (f0) atomicOr(&s_flip[x0 >> 5], 1u << (x0 & 31));
-          if (f1) atomicOr(&s_flip[x1 >> 5], 1u << (x1 & 31));
-          qh += 64;
-          qn -= 64;
+        if (qn >= QD) {
+          int x[QD / 32];
+          uint32_t f[QD / 32];
+#pragma unroll
+          for (int i = 0; i < QD / 32; ++i) {
+            x[i] = q[(qh + 32 * i + lane) & (QC - 1)];
+            f[i] = draw(x[i]);
+          }
+#pragma unroll
+          for (int i = 0; i < QD / 32; ++i)
+            if (f[i]) atomicOr(&s_flip[x[i] >> 5], 1u << (x[i] & 31));
+          qh += QD;
+          qn -= QD;
           __syncwarp();
         }
       }
@@ -2142,15 +2149,18 @@ cudaError_t launch_phase31(int shape, const SweepArgs& a3, const SweepArgs& a1, 
     case 6:
       phase31_kernel<shape_of(6).wpr, shape_of(6).th, shape_of(6).h><<<ntiles, 32 * shape_of(6).wpr, 0, st>>>(a3, a1);
       return cudaGetLastError();
+    case 7:
+      phase31_kernel<shape_of(7).wpr, shape_of(7).th, shape_of(7).h><<<ntiles, 32 * shape_of(7).wpr, 0, st>>>(a3, a1);
+      return cudaGetLastError();
   }
   return cudaErrorInvalidValue;
 }
 
-bool batch_fused_supported(int shape) {
-  if (shape < 0 || shape >= kNumShapes) return false;
-  const TileShape ts = shape_of(shape);
-  return ts.th == 32 * ts.h;
+bool phase31_supported(int shape) {
+  return shape >= 0 && shape < kNumShapes && shape_of(shape).th == 32 * shape_of(shape).h;
 }
+
+bool batch_fused_supported(int shape) { return phase31_supported(shape) && shape_of(shape).th >= 64; }
 
 cudaError_t launch_batch_fused(int shape, const BatchArgs& b, int ntiles, int nsweeps, cudaStream_t st) {
   if (ntiles <= 0 || nsweeps <= 0) return cudaSuccess;
