@@ -18,6 +18,38 @@ enum DeviceError : int {
   kErrBarrierTimeout = 5,  // a grid barrier of the fused batch kernel did not open within its time limit
 };
 
+#ifdef __CUDACC__
+// Programmatic dependent launch. A kernel launched by launch_after may start
+// once every CTA of the kernel before it in the stream has called
+// start_next() (or ended), and takes part in the stream's order by calling
+// after_previous() before anything else: it waits until everything before it
+// has finished and its writes are visible. What overlaps is the launch
+// itself, which small lattices pay for three or four times a sweep; no work
+// moves. Without the attribute on the launch, or after any other kind of
+// work, the wait returns at once. Kernels whose CTAs are few and long call
+// start_next() near their end: the next kernel's CTAs are placed when it is
+// called, and from the start they would be placed around this kernel's, two
+// or three to one SM and none to another (L = 2048 56 -> 74 us a sweep).
+__device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                         const A&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 // A tile shape: TW = 32*WPR columns by TH rows. Phase 1 runs one warp per
 // 32-column band (32 * WPR threads); in phase 3 each thread owns one 32-site
 // word column of an H-row strip of the tile (WPR * TH/H threads per tile).

@@ -956,6 +956,7 @@ __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const Sweep
     const int r = s_broot[j];
     bs[j] = r >= 0 ? (uint16_t)slot_of(s_bmask, s_pre, r) : (uint16_t)0xFFFFu;
   }
+  if (!BATCH) start_next();
   // labels and border marks for phase 3
   {
     const uint4* src = reinterpret_cast<const uint4*>(par);
@@ -986,6 +987,7 @@ constexpr int phase1_min_blocks() {
 template <int WPR, int TH, int H, bool BATCH>
 __global__ void __launch_bounds__(32 * WPR, phase1_min_blocks<32 * WPR>())
     phase1_kernel(const SweepArgs a0, const BatchArgs bat) {
+  if (!BATCH) after_previous();
   __shared__ P1Shared<WPR, TH, H> S;
   phase1_body<WPR, TH, H, BATCH>(S, a0, bat, blockIdx.x, 0);
 }
@@ -1092,9 +1094,12 @@ constexpr int phase2_threads() {
 }
 template <int WPR, int TH, int H, bool BATCH>
 __global__ void __launch_bounds__(phase2_threads<TH, 32 * WPR>(), 2048 / phase2_threads<TH, 32 * WPR>()) phase2_kernel(const SweepArgs a0, const BatchArgs bat) {
+  if (!BATCH && !a0.draws_out) start_next();  // else when the draws are done: they are the longer part
+  if (!BATCH) after_previous();
   using Tl = Tile<WPR, TH, H>;
   if (!BATCH && a0.draws_out && threadIdx.x >= TH + Tl::TW) {
     draw_next_bonds<WPR, TH, H>(a0, blockIdx.x, threadIdx.x - (TH + Tl::TW), 0, draw_split<Tl::RW>());
+    start_next();
     return;
   }
   phase2_body<WPR, TH, H, BATCH>(a0, bat, blockIdx.x, 0);
@@ -1153,13 +1158,16 @@ __device__ __forceinline__ void resolve_body(const SweepArgs& a0, const BatchArg
 constexpr int kResolveThreads = 128;
 template <int WPR, int TH, int H, bool BATCH>
 __global__ void __launch_bounds__(kResolveThreads + 32 * kDrawWarps, 10) resolve_kernel(const SweepArgs a0, const BatchArgs bat) {
+  if (!BATCH) after_previous();
   using Tl = Tile<WPR, TH, H>;
   if (threadIdx.x >= kResolveThreads) {
     if (!BATCH && a0.draws_out)
       draw_next_bonds<WPR, TH, H>(a0, blockIdx.x, threadIdx.x - kResolveThreads, draw_split<Tl::RW>(), Tl::RW);
+    start_next();
     return;
   }
   resolve_body<WPR, TH, H, BATCH>(a0, bat, blockIdx.x, 0, kResolveThreads);
+  if (!BATCH && !a0.draws_out) start_next();  // the draws end later than the walks
 }
 
 // ================================================================ phase 3
@@ -1187,7 +1195,8 @@ struct P3Shared {
 
 // Returns false when the labels' bulk copy did not land (the CTA's shared
 // memory may still be written by it: the caller must not reuse it).
-template <int WPR, int TH, int H, int MODE, bool BATCH>
+// LAST: nothing of the launch follows, so the next one may start before E and M.
+template <int WPR, int TH, int H, int MODE, bool BATCH, bool LAST = false>
 __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint32_t* s_size, const SweepArgs& a0,
                                             const BatchArgs& bat, int T, int ksweep) {
   using Tl = Tile<WPR, TH, H>;
@@ -1485,6 +1494,7 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
       return spin_bytes4(__funnelshift_r(s_snew[y][ww], ww + 1 < WPR ? s_snew[y][ww + 1] : 0u, x & 31) & 0xFu);
     });
 
+  if (LAST && !HIST) start_next();
   // ---- E and M of the new state (C10)
   int eloc = 0, mloc = 0;
 #pragma unroll
@@ -1570,6 +1580,7 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
       atomicAdd(reinterpret_cast<unsigned long long*>(a.em + 1), (unsigned long long)m2);
     }
   }
+  if (LAST && HIST) start_next();
   if (HIST)
     for (int i = tid; i < 34; i += NT)
       if (s_hist[i]) atomicAdd(reinterpret_cast<unsigned long long*>(a.hist + i), s_hist[i]);
@@ -1579,15 +1590,17 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
 template <int WPR, int TH, int H, int MODE, bool BATCH>
 __global__ void __launch_bounds__(WPR * (TH / H), strip_min_blocks<WPR * (TH / H), H>())
     phase3_kernel(const SweepArgs a0, const BatchArgs bat) {
+  if (!BATCH) after_previous();
   __shared__ P3Shared<WPR, TH, H, MODE> S;
   extern __shared__ __align__(16) uint32_t s_size[];  // HIST: [TH * TW / 2], two 16-bit sizes a word
-  phase3_body<WPR, TH, H, MODE, BATCH>(S, s_size, a0, bat, blockIdx.x, 0);
+  phase3_body<WPR, TH, H, MODE, BATCH, !BATCH>(S, s_size, a0, bat, blockIdx.x, 0);
 }
 
 // ================================================================ phase 4
 
 template <int WPR, int TH, int H>
 __global__ void phase4_kernel(const SweepArgs a) {
+  after_previous();
   using T = Tile<WPR, TH, H>;
   constexpr int MS = T::MS;
   __shared__ unsigned long long s_hist[34];
@@ -1608,6 +1621,7 @@ __global__ void phase4_kernel(const SweepArgs a) {
     }
   }
   __syncthreads();
+  start_next();
   if (threadIdx.x < 34 && s_hist[threadIdx.x])
     atomicAdd(reinterpret_cast<unsigned long long*>(a.hist + threadIdx.x), s_hist[threadIdx.x]);
 }
@@ -1726,6 +1740,7 @@ __global__ void __launch_bounds__(32 * WPR, band_min_blocks<32 * WPR>())
 template <int WPR, int TH, int H>
 __global__ void __launch_bounds__(32 * WPR, band_min_blocks<32 * WPR>())
     phase31_kernel(const SweepArgs a3, const SweepArgs a1) {
+  after_previous();
   using Tl = Tile<WPR, TH, H>;
   constexpr int NT = 32 * WPR, RPL = TH / 32, NHE = TH / 32, NH = TH / 32 + Tl::TW / 32;
   static_assert(Tl::NT == NT, "phases 1 and 3 run the same block");
@@ -1784,6 +1799,7 @@ cudaError_t launch_fused_shape(const BatchArgs& b, int ntiles, int nsweeps, cuda
 template <int WPR, int TH, int H, bool ALIGNED>
 __global__ void __launch_bounds__(32 * WPR, band_min_blocks<32 * WPR>())
     potts_phase1_kernel(const SweepArgs a) {
+  after_previous();
   __shared__ P1Shared<WPR, TH, H> S;
   phase1_body<WPR, TH, H, false, false, true, ALIGNED>(S, a, BatchArgs{}, blockIdx.x, 0);
 }
@@ -1813,6 +1829,7 @@ struct PottsP3Shared {
 // ALIGNED: L is a multiple of 16 (every four sites are one aligned store).
 template <int WPR, int TH, int H, bool ALIGNED>
 __global__ void __launch_bounds__(kPottsP3Threads) potts_phase3_kernel(const SweepArgs a) {
+  after_previous();
   using Tl = Tile<WPR, TH, H>;
   constexpr int TW = Tl::TW, NT = kPottsP3Threads, NB = Tl::NB, MS = Tl::MS, RW = Tl::RW;
   constexpr int G = TW / 4;  // four-site groups per row
@@ -1916,6 +1933,7 @@ __global__ void __launch_bounds__(kPottsP3Threads) potts_phase3_kernel(const Swe
       return __funnelshift_r(row[q], q + 1 < G ? row[q + 1] : 0u, 8 * (x & 3));
     });
 
+  start_next();
   // ---- E and M of the new states: east and south edge of every site
   long long e = 0, m = 0;
   for (int i = tid; i < TH * G; i += NT) {
@@ -2015,34 +2033,39 @@ cudaError_t launch_all(int which, const SweepArgs& a, int mode, uint8_t* out, cu
                        const BatchArgs* batch, int batch_tiles) {
   using T = Tile<WPR, TH, H>;
   const int ntiles = batch ? batch_tiles : a.g.tiles_x * a.g.tiles_y;
+  cudaError_t e = cudaSuccess;
   switch (which) {
     case 1:
-      phase1_kernel<WPR, TH, H, false><<<ntiles, 32 * WPR, 0, st>>>(a, BatchArgs{});
+      e = launch_after(phase1_kernel<WPR, TH, H, false>, ntiles, 32 * WPR, 0, st, a, BatchArgs{});
       break;
     case 2:
       {
         const int xd = a.draws_out ? 32 * kDrawWarps : 0;  // the warps that draw the next sweep's bonds
-        phase2_kernel<WPR, TH, H, false><<<ntiles, TH + T::TW + xd, 0, st>>>(a, BatchArgs{});
-        resolve_kernel<WPR, TH, H, false><<<ntiles, kResolveThreads + xd, 0, st>>>(a, BatchArgs{});
+        e = launch_after(phase2_kernel<WPR, TH, H, false>, ntiles, TH + T::TW + xd, 0, st, a, BatchArgs{});
+        if (e == cudaSuccess)
+          e = launch_after(resolve_kernel<WPR, TH, H, false>, ntiles, kResolveThreads + xd, 0, st, a, BatchArgs{});
       }
       break;
     case 3:
       if (mode == 0) {
-        phase3_kernel<WPR, TH, H, 0, false><<<ntiles, T::NT, 0, st>>>(a, BatchArgs{});
+        e = launch_after(phase3_kernel<WPR, TH, H, 0, false>, ntiles, T::NT, 0, st, a, BatchArgs{});
       } else if (mode == 1) {
         const size_t dyn = (size_t)TH * T::TW * sizeof(uint16_t);
         static bool attr_done = false;
         if (!attr_done) {
-          cudaError_t e = cudaFuncSetAttribute(phase3_kernel<WPR, TH, H, 1, false>,
+          e = cudaFuncSetAttribute(phase3_kernel<WPR, TH, H, 1, false>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
           if (e != cudaSuccess) return e;
           attr_done = true;
         }
-        phase3_kernel<WPR, TH, H, 1, false><<<ntiles, T::NT, dyn, st>>>(a, BatchArgs{});
+        e = launch_after(phase3_kernel<WPR, TH, H, 1, false>, ntiles, T::NT, dyn, st, a, BatchArgs{});
       } else {
-        phase3_kernel<WPR, TH, H, 2, false><<<ntiles, T::NT, 0, st>>>(a, BatchArgs{});
+        e = launch_after(phase3_kernel<WPR, TH, H, 2, false>, ntiles, T::NT, 0, st, a, BatchArgs{});
       }
       break;
+    // (the batch's launches are replayed from a graph, whose launches cost
+    // little: dependent launches measured 3 % faster at 2 replicas and 1.5 %
+    // slower on the benchmark's 256)
     case 11:
       phase1_kernel<WPR, TH, H, true><<<ntiles, 32 * WPR, 0, st>>>(a, *batch);
       break;
@@ -2055,14 +2078,14 @@ cudaError_t launch_all(int which, const SweepArgs& a, int mode, uint8_t* out, cu
       break;
     case 4: {
       const long long total = (long long)ntiles * T::MS;
-      phase4_kernel<WPR, TH, H><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(a);
+      e = launch_after(phase4_kernel<WPR, TH, H>, (unsigned)((total + 255) / 256), 256, 0, st, a);
       break;
     }
     case 5:
       export_bonds_kernel<WPR, TH, H><<<grid_for((long long)a.g.L * a.g.L, 256), 256, 0, st>>>(a, out);
       break;
   }
-  return cudaGetLastError();
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 template <int V>
@@ -2115,17 +2138,15 @@ cudaError_t launch_export_bonds(int shape, const SweepArgs& a, uint8_t* out, cud
 cudaError_t launch_potts_phase1(const SweepArgs& a, cudaStream_t st) {
   constexpr TileShape ts = shape_of(kPottsShape);
   const int n = a.g.tiles_x * a.g.tiles_y;
-  if (a.g.aligned16) potts_phase1_kernel<ts.wpr, ts.th, ts.h, true><<<n, 32 * ts.wpr, 0, st>>>(a);
-  else potts_phase1_kernel<ts.wpr, ts.th, ts.h, false><<<n, 32 * ts.wpr, 0, st>>>(a);
-  return cudaGetLastError();
+  return a.g.aligned16 ? launch_after(potts_phase1_kernel<ts.wpr, ts.th, ts.h, true>, n, 32 * ts.wpr, 0, st, a)
+                       : launch_after(potts_phase1_kernel<ts.wpr, ts.th, ts.h, false>, n, 32 * ts.wpr, 0, st, a);
 }
 
 cudaError_t launch_potts_phase3(const SweepArgs& a, cudaStream_t st) {
   constexpr TileShape ts = shape_of(kPottsShape);
   const int n = a.g.tiles_x * a.g.tiles_y;
-  if (a.g.aligned16) potts_phase3_kernel<ts.wpr, ts.th, ts.h, true><<<n, kPottsP3Threads, 0, st>>>(a);
-  else potts_phase3_kernel<ts.wpr, ts.th, ts.h, false><<<n, kPottsP3Threads, 0, st>>>(a);
-  return cudaGetLastError();
+  return a.g.aligned16 ? launch_after(potts_phase3_kernel<ts.wpr, ts.th, ts.h, true>, n, kPottsP3Threads, 0, st, a)
+                       : launch_after(potts_phase3_kernel<ts.wpr, ts.th, ts.h, false>, n, kPottsP3Threads, 0, st, a);
 }
 
 cudaError_t launch_batch_phase(int shape, int which, const BatchArgs& b, int ntiles, cudaStream_t st) {
@@ -2140,18 +2161,29 @@ cudaError_t launch_batch_advance(const BatchArgs& b, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+namespace {
+template <int V>
+cudaError_t launch_phase31_shape(const SweepArgs& a3, const SweepArgs& a1, cudaStream_t st) {
+  constexpr TileShape ts = shape_of(V);
+  const auto kernel = phase31_kernel<ts.wpr, ts.th, ts.h>;
+  const int n = a3.g.tiles_x * a3.g.tiles_y;
+  // One to three tiles an SM: a plain launch. The resolve pass before it ends
+  // CTA by CTA with its draws, and tiles placed meanwhile crowd the SMs that
+  // ended first (L = 1024, 256 tiles: 40 -> 45 us a sweep). Fewer tiles have
+  // an SM each either way, more even out (256: 37 -> 30, 2048: 56 -> 51).
+  if (n > 152 && n <= 3 * 152) {
+    kernel<<<n, 32 * ts.wpr, 0, st>>>(a3, a1);
+    return cudaGetLastError();
+  }
+  return launch_after(kernel, n, 32 * ts.wpr, 0, st, a3, a1);
+}
+}  // namespace
+
 cudaError_t launch_phase31(int shape, const SweepArgs& a3, const SweepArgs& a1, cudaStream_t st) {
-  const int ntiles = a3.g.tiles_x * a3.g.tiles_y;
   switch (shape) {
-    case 4:
-      phase31_kernel<shape_of(4).wpr, shape_of(4).th, shape_of(4).h><<<ntiles, 32 * shape_of(4).wpr, 0, st>>>(a3, a1);
-      return cudaGetLastError();
-    case 6:
-      phase31_kernel<shape_of(6).wpr, shape_of(6).th, shape_of(6).h><<<ntiles, 32 * shape_of(6).wpr, 0, st>>>(a3, a1);
-      return cudaGetLastError();
-    case 7:
-      phase31_kernel<shape_of(7).wpr, shape_of(7).th, shape_of(7).h><<<ntiles, 32 * shape_of(7).wpr, 0, st>>>(a3, a1);
-      return cudaGetLastError();
+    case 4: return launch_phase31_shape<4>(a3, a1, st);
+    case 6: return launch_phase31_shape<6>(a3, a1, st);
+    case 7: return launch_phase31_shape<7>(a3, a1, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -230,6 +230,8 @@ __device__ __forceinline__ float to_binary32(double v) {
 // The projections in binary64 and, for the bond kernel's first test, rounded
 // to binary32.
 __global__ void phi4_project_kernel(const F4* phi, double* a, float* af, int64_t n, Dir d, uint32_t* top) {
+  sw::start_next();
+  sw::after_previous();
   uint32_t big = 0u;  // high word of the largest |component|
   GRID_LOOP(x, n) {
     const F4 f = phi[x];
@@ -268,6 +270,8 @@ template <int B0, int B1, int B2, int B3, int NT>
 __global__ void __launch_bounds__(NT)
     phi4_brick_kernel(const double* a, const float* af, uint8_t* bonds, int* par, int L, double k4, uint32_t t,
                       sw::KeySchedule ks, int* err) {
+  sw::start_next();
+  sw::after_previous();
   constexpr int V = B0 * B1 * B2 * B3, S1 = B0, S2 = B0 * B1, S3 = B0 * B1 * B2;
   __shared__ float s_af[V];
   __shared__ int s_par[V];
@@ -388,6 +392,8 @@ constexpr int kUniteWarps = 4, kUniteCap = 2 * 128;
 template <int ROWS>
 __global__ void __launch_bounds__(32 * kUniteWarps)
     phi4_unite_kernel(const uint8_t* bonds, int* par, int L, int64_t n, int* err) {
+  sw::start_next();
+  sw::after_previous();
   __shared__ int2 s_list[kUniteWarps][kUniteCap];
   const int lane = threadIdx.x & 31;
   int2* const list = s_list[threadIdx.x >> 5];
@@ -443,6 +449,8 @@ constexpr int kRootWarps = 4;
 template <int ROWS>
 __global__ void __launch_bounds__(32 * kRootWarps)
     phi4_roots_kernel(const uint8_t* bonds, int* par, int64_t n, uint32_t t, sw::KeySchedule ks, int* err) {
+  sw::start_next();
+  sw::after_previous();
   __shared__ uint8_t s_list[kRootWarps][32 * ROWS];
   static_assert(32 * ROWS <= 256, "8-bit entries");
   const int lane = threadIdx.x & 31;
@@ -477,10 +485,14 @@ __global__ void __launch_bounds__(32 * kRootWarps)
 }
 
 __global__ void phi4_labels_kernel(const int* par, int* out, int64_t n) {
+  sw::start_next();
+  sw::after_previous();
   GRID_LOOP(x, n) out[x] = par[par[x] & kSiteMask] & kSiteMask;
 }
 
 __global__ void phi4_reflect_kernel(F4* phi, const double* a, const int* par, int64_t n, Dir d) {
+  sw::start_next();
+  sw::after_previous();
   GRID_LOOP(x, n) {
     if (par[par[x] & kSiteMask] >= 0) continue;  // the cluster's decision: not flipped
     // a (-2 r_c) is the same product as (-2 a) r_c, both factors exact (unless
@@ -578,6 +590,8 @@ __device__ void observe_binary64(const F4* phi, int L, int64_t n, int64_t x0, in
 }
 
 __global__ void phi4_observe_kernel(const F4* phi, int L, int64_t n, double* out /* E, M0..M3 */) {
+  sw::start_next();
+  sw::after_previous();
   double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   observe_binary64(phi, L, n, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, v);
   block_add5(v, out);
@@ -607,6 +621,8 @@ template <bool PROJECT>
 __global__ void __launch_bounds__(kObserveThreads)
     phi4_observe_fixed_kernel(const F4* phi, int L, int64_t n, const uint32_t* top, int steps, double* out, double* a,
                               float* af, Dir d, uint32_t* next_top) {
+  sw::start_next();
+  sw::after_previous();
   uint32_t big = 0u;
   auto project = [&](const F4& f, size_t x) {
     const double v = proj(f, d);
@@ -801,17 +817,17 @@ template <int B0, int B1, int B2, int B3, int NT>
 void launch_brick(sw_phi4* h) {
   const int L = h->L;
   const unsigned g = (unsigned)((L + B0 - 1) / B0) * ((L + B1 - 1) / B1) * ((L + B2 - 1) / B2) * ((L + B3 - 1) / B3);
-  phi4_brick_kernel<B0, B1, B2, B3, NT>
-      <<<g, NT, 0, h->stream>>>(h->a, h->af, h->bonds, h->par, L, 4.0 * h->kappa, (uint32_t)h->t, h->ks, h->err);
+  sw::launch_after(phi4_brick_kernel<B0, B1, B2, B3, NT>, g, NT, 0, h->stream, h->a, h->af, h->bonds, h->par, L,
+                   4.0 * h->kappa, (uint32_t)h->t, h->ks, h->err);
 }
 
 template <int UNITE_ROWS, int ROOT_ROWS>
 void launch_merge(sw_phi4* h) {
   const int64_t u = 32 * kUniteWarps * UNITE_ROWS, r = 32 * kRootWarps * ROOT_ROWS;
-  phi4_unite_kernel<UNITE_ROWS><<<(unsigned)((h->n + u - 1) / u), 32 * kUniteWarps, 0, h->stream>>>(
-      h->bonds, h->par, h->L, h->n, h->err);
-  phi4_roots_kernel<ROOT_ROWS><<<(unsigned)((h->n + r - 1) / r), 32 * kRootWarps, 0, h->stream>>>(
-      h->bonds, h->par, h->n, (uint32_t)h->t, h->ks, h->err);
+  sw::launch_after(phi4_unite_kernel<UNITE_ROWS>, (unsigned)((h->n + u - 1) / u), 32 * kUniteWarps, 0, h->stream,
+                   h->bonds, h->par, h->L, h->n, h->err);
+  sw::launch_after(phi4_roots_kernel<ROOT_ROWS>, (unsigned)((h->n + r - 1) / r), 32 * kRootWarps, 0, h->stream,
+                   h->bonds, h->par, h->n, (uint32_t)h->t, h->ks, h->err);
 }
 
 // The direction of update t and, on large lattices, its cleared range word.
@@ -823,8 +839,8 @@ int begin_update(sw_phi4* h, int64_t t, Dir& d) {
 
 // Projections of update t on direction d.
 void project(sw_phi4* h, const Dir& d) {
-  phi4_project_kernel<<<grid_of(h->n), 256, 0, h->stream>>>(h->phi, h->a, h->af, h->n, d,
-                                                            h->n >= kLargeSites ? h->top + (h->t & 1) : nullptr);
+  sw::launch_after(phi4_project_kernel, grid_of(h->n), 256, 0, h->stream, h->phi, h->a, h->af, h->n, d,
+                   h->n >= kLargeSites ? h->top + (h->t & 1) : nullptr);
 }
 
 // Bonds, clusters and flips of update t from its projections.
@@ -919,14 +935,14 @@ int sw_phi4_sweep(sw_phi4* h, int32_t n) {
   Dir d, next{};
   rc = begin_update(h, h->t, d);
   if (rc != SW_OK) return rc;
+  F_CUDA(cudaMemsetAsync(h->obs + 5 * (h->t - h->t_base), 0, (size_t)n * 5 * sizeof(double), h->stream), "trace rows");
   project(h, d);
   for (int32_t k = 0; k < n; ++k) {
     rc = clusters(h);
     if (rc != SW_OK) return rc;
     double* o = h->obs + 5 * (h->t - h->t_base);
     uint32_t* const top = h->top + (h->t & 1);
-    F_CUDA(cudaMemsetAsync(o, 0, 5 * sizeof(double), h->stream), "trace row");
-    phi4_reflect_kernel<<<g, 256, 0, h->stream>>>(h->phi, h->a, h->par, h->n, d);
+    sw::launch_after(phi4_reflect_kernel, g, 256, 0, h->stream, h->phi, h->a, h->par, h->n, d);
     // E and M, with the next update's projections unless the call ends here
     // (the caller may change the field before the next one)
     const bool more = k + 1 < n;
@@ -935,13 +951,13 @@ int sw_phi4_sweep(sw_phi4* h, int32_t n) {
       if (rc != SW_OK) return rc;
     }
     if (large && more)
-      phi4_observe_fixed_kernel<true><<<og, kObserveThreads, 0, h->stream>>>(
-          h->phi, L, h->n, top, kObserveSteps, o, h->a, h->af, next, h->top + ((h->t + 1) & 1));
+      sw::launch_after(phi4_observe_fixed_kernel<true>, og, kObserveThreads, 0, h->stream, h->phi, L, h->n, top,
+                       kObserveSteps, o, h->a, h->af, next, h->top + ((h->t + 1) & 1));
     else if (large)
-      phi4_observe_fixed_kernel<false>
-          <<<og, kObserveThreads, 0, h->stream>>>(h->phi, L, h->n, top, kObserveSteps, o, nullptr, nullptr, d, nullptr);
+      sw::launch_after(phi4_observe_fixed_kernel<false>, og, kObserveThreads, 0, h->stream, h->phi, L, h->n, top,
+                       kObserveSteps, o, nullptr, nullptr, d, nullptr);
     else
-      phi4_observe_kernel<<<g, 256, 0, h->stream>>>(h->phi, L, h->n, o);
+      sw::launch_after(phi4_observe_kernel, g, 256, 0, h->stream, h->phi, L, h->n, o);
     F_CUDA(cudaGetLastError(), "phi4 reflect launch");
     h->t += 1;
     if (more && !large) project(h, next);
@@ -1005,8 +1021,8 @@ int sw_phi4_labels(sw_phi4* h, int32_t* out, int32_t out_is_device) {
   if (rc != SW_OK) return rc;
   // host labels pass through the projections' buffer (8 bytes a site), done with here
   int32_t* const dst = out_is_device ? out : reinterpret_cast<int32_t*>(h->a);
-  phi4_labels_kernel<<<grid_of(h->n), 256, 0, h->stream>>>(h->par, dst, h->n);
-  F_CUDA(cudaGetLastError(), "phi4 labels launch");
+  F_CUDA(sw::launch_after(phi4_labels_kernel, grid_of(h->n), 256, 0, h->stream, h->par, dst, h->n),
+         "phi4 labels launch");
   if (out_is_device) return SW_OK;
   F_CUDA(cudaMemcpyAsync(out, dst, (size_t)h->n * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream), "labels copy");
   return check_phi4(h);
