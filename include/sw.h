@@ -130,7 +130,7 @@ int sw_destroy(sw_lattice* h);
  * sweep E and M (C10), and the C11 statistics if enabled, are appended to
  * the device-side trace. Errors: SW_EINVAL (n < 0), SW_ENOMEM (trace
  * growth), SW_ECUDA. Device-side failures are reported by the next call that
- * synchronises. A lattice with L <= 160 (208 for n >= 4) and statistics off runs all n
+ * synchronises. A lattice with L <= 160 (144 for n = 1) and statistics off runs all n
  * sweeps in one CTA-sized launch (the whole lattice in shared memory)
  * unless the environment variable SW_TILE_SHAPE was set at sw_create, which
  * keeps it on the tiled path; the results are the same. Between the sweeps
@@ -221,7 +221,7 @@ int sw_bonds(sw_lattice* h, uint8_t* out_host);
  * 0 = bonds + tile-local clusters, 1 = cross-tile merge, 2 = flips + E/M,
  * 3 = cluster statistics, 4 = flips + E/M of a sweep together with the bonds
  * and tile-local clusters of the next sweep of the same call (one launch,
- * on the 128x64 and 128x128 tile shapes with statistics off; a call's last
+ * on the 128x32, 128x64 and 128x128 tile shapes with statistics off; a call's last
  * sweep runs phase 2 alone). Not part of the paper: measurement support. */
 #define SW_TIMING_PHASES 5
 int sw_timing(sw_lattice* h, int32_t enable);
@@ -492,7 +492,7 @@ int sw_shape_info(int32_t shape, int32_t* tile_w, int32_t* tile_h, int32_t* stri
 int sw_tune_shape(int32_t log2_bucket, int32_t shape);
 
 /* The tile shape index a lattice was created with (its tiled path; sides up
- * to 160 (208) run whole sweeps in one CTA unless SW_TILE_SHAPE is set). */
+ * to 160 run whole sweeps in one CTA unless SW_TILE_SHAPE is set). */
 int sw_lattice_shape(sw_lattice* h, int32_t* shape);
 
 /* Message of the last failed call on this thread ("" if none). */

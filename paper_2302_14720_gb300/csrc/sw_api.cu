@@ -76,7 +76,7 @@ int shape_for(int L, bool lattice) {
   });
   const int t = g_tuned[bucket_of(L)].load();
   if (t >= 0) return t;
-  if (L <= 64) return 2;
+  if (!lattice && L <= 64) return 2;
   // A lone lattice of side <= 1024 has at most 128 tiles of 128 x 64, less
   // than one wave of 152 SMs; with 128 x 32 tiles twice as many CTAs share
   // each phase's latency, and in phase 3 a thread has one row word (one-row

@@ -195,15 +195,15 @@ cudaError_t launch_batch_fused(int shape, const BatchArgs& b, int ntiles, int ns
 // so 16-bit parents index every site.
 constexpr int kSmallMaxL = 181;
 // sw_sweep takes the one-CTA path (any L <= 256 fits) up to kSmallSweepMaxL,
-// and up to kSmallChainMaxL in calls of four sweeps or more: a sweep costs the
-// CTA less than the tiled path's launches up to about L = 220, its first one
-// twice that. Us per sweep of a 100-sweep call (with one union-find over all
-// runs, before the segments): L = 64 9.0 (15.2), 100 14.5 (37.7), 144 20.7
-// (67.0); one CTA / tiled: 181 33 / 49, 208 39 / 46, 256 57 / 46. One-sweep
-// calls with their read-back: L = 160 80 / 84, 181 97 / 84.
+// for calls of one sweep up to kSmallCallMaxL: a sweep costs the CTA less
+// than the tiled path's launches up to there, its first one twice that. Us
+// per sweep of a 100-sweep call (with one union-find over all runs, before
+// the segments): L = 64 9.0 (15.2), 100 14.5 (37.7), 144 20.7 (67.0); one
+// CTA / tiled: 160 24 / 30, 181 33 / 31, 256 57 / 30. One-sweep calls with
+// their read-back: L = 144 76 / 73, 160 80 / 73.
 constexpr int kSmallSweepMaxL = 160;
-constexpr int kSmallChainMaxL = 208;
-inline bool small_sweep(int L, int n) { return L <= kSmallSweepMaxL || (L <= kSmallChainMaxL && n >= 4); }
+constexpr int kSmallCallMaxL = 144;
+inline bool small_sweep(int L, int n) { return L <= kSmallCallMaxL || (L <= kSmallSweepMaxL && n > 1); }
 struct SmallArgs {
   int L;
   uint32_t thr;    // C3
@@ -229,13 +229,14 @@ cudaError_t run_label_equivalence(const uint8_t* bonds, int L, int32_t* lab, int
 // Debug: expand the stored bond bits into uint8 [L][L] (bit0 east, bit1 south).
 cudaError_t launch_export_bonds(int shape, const SweepArgs& a, uint8_t* out, cudaStream_t st);
 
-// q-state Potts sweeps (§6) on the 128x64 tile shape: phase 1 bonds equal
-// states, phase 2 (launch_phase2) is the Ising one with resolve drawing each
-// border cluster's new state into tb.nval, and phase 3 assigns the states and
-// sums E, M. Labels come from launch_phase3's labels mode. a.q >= 2.
-constexpr int kPottsShape = 6;
+// q-state Potts sweeps (§6) on the 128x64 tile shape, or 128x32 up to L = 1024
+// for the same reason as the Ising lattices: phase 1 bonds equal states,
+// phase 2 (launch_phase2) is the Ising one with resolve drawing each border
+// cluster's new state into tb.nval, and phase 3 assigns the states and sums
+// E, M. Labels come from launch_phase3's labels mode. a.q >= 2.
+inline int potts_shape(int L) { return L <= 1024 ? 7 : 6; }
 constexpr int kPottsPad = 64;  // bytes of the state buffer past its last site (phase 1 loads whole row words)
-cudaError_t launch_potts_phase1(const SweepArgs& a, cudaStream_t st);
-cudaError_t launch_potts_phase3(const SweepArgs& a, cudaStream_t st);
+cudaError_t launch_potts_phase1(int shape, const SweepArgs& a, cudaStream_t st);
+cudaError_t launch_potts_phase3(int shape, const SweepArgs& a, cudaStream_t st);
 
 }  // namespace sw

@@ -1804,7 +1804,11 @@ __global__ void __launch_bounds__(32 * WPR, band_min_blocks<32 * WPR>())
   phase1_body<WPR, TH, H, false, false, true, ALIGNED>(S, a, BatchArgs{}, blockIdx.x, 0);
 }
 
-constexpr int kPottsP3Threads = 256;  // threads per tile of the Potts phase 3
+// Threads per tile of the Potts phase 3: one to every row word, 256 at most.
+template <int WPR, int TH>
+constexpr int potts_p3_threads() {
+  return WPR * TH < 256 ? WPR * TH : 256;
+}
 
 template <int WPR, int TH, int H, int NT>
 struct PottsP3Shared {
@@ -1828,10 +1832,10 @@ struct PottsP3Shared {
 // configuration are summed in int64.
 // ALIGNED: L is a multiple of 16 (every four sites are one aligned store).
 template <int WPR, int TH, int H, bool ALIGNED>
-__global__ void __launch_bounds__(kPottsP3Threads) potts_phase3_kernel(const SweepArgs a) {
+__global__ void __launch_bounds__(potts_p3_threads<WPR, TH>()) potts_phase3_kernel(const SweepArgs a) {
   after_previous();
   using Tl = Tile<WPR, TH, H>;
-  constexpr int TW = Tl::TW, NT = kPottsP3Threads, NB = Tl::NB, MS = Tl::MS, RW = Tl::RW;
+  constexpr int TW = Tl::TW, NT = potts_p3_threads<WPR, TH>(), NB = Tl::NB, MS = Tl::MS, RW = Tl::RW;
   constexpr int G = TW / 4;  // four-site groups per row
   static_assert(RW % NT == 0, "whole rounds of row words");
   __shared__ PottsP3Shared<WPR, TH, H, NT> S;
@@ -2135,18 +2139,25 @@ cudaError_t launch_export_bonds(int shape, const SweepArgs& a, uint8_t* out, cud
   return dispatch(shape, 5, a, 0, out, st);
 }
 
-cudaError_t launch_potts_phase1(const SweepArgs& a, cudaStream_t st) {
-  constexpr TileShape ts = shape_of(kPottsShape);
+namespace {
+template <int V>
+cudaError_t launch_potts(int phase, const SweepArgs& a, cudaStream_t st) {
+  constexpr TileShape ts = shape_of(V);
+  constexpr int W = ts.wpr, TH = ts.th, H = ts.h, N1 = 32 * W, N3 = potts_p3_threads<W, TH>();
   const int n = a.g.tiles_x * a.g.tiles_y;
-  return a.g.aligned16 ? launch_after(potts_phase1_kernel<ts.wpr, ts.th, ts.h, true>, n, 32 * ts.wpr, 0, st, a)
-                       : launch_after(potts_phase1_kernel<ts.wpr, ts.th, ts.h, false>, n, 32 * ts.wpr, 0, st, a);
+  if (phase == 1)
+    return a.g.aligned16 ? launch_after(potts_phase1_kernel<W, TH, H, true>, n, N1, 0, st, a)
+                         : launch_after(potts_phase1_kernel<W, TH, H, false>, n, N1, 0, st, a);
+  return a.g.aligned16 ? launch_after(potts_phase3_kernel<W, TH, H, true>, n, N3, 0, st, a)
+                       : launch_after(potts_phase3_kernel<W, TH, H, false>, n, N3, 0, st, a);
 }
+}  // namespace
 
-cudaError_t launch_potts_phase3(const SweepArgs& a, cudaStream_t st) {
-  constexpr TileShape ts = shape_of(kPottsShape);
-  const int n = a.g.tiles_x * a.g.tiles_y;
-  return a.g.aligned16 ? launch_after(potts_phase3_kernel<ts.wpr, ts.th, ts.h, true>, n, kPottsP3Threads, 0, st, a)
-                       : launch_after(potts_phase3_kernel<ts.wpr, ts.th, ts.h, false>, n, kPottsP3Threads, 0, st, a);
+cudaError_t launch_potts_phase1(int shape, const SweepArgs& a, cudaStream_t st) {
+  return shape == 6 ? launch_potts<6>(1, a, st) : shape == 7 ? launch_potts<7>(1, a, st) : cudaErrorInvalidValue;
+}
+cudaError_t launch_potts_phase3(int shape, const SweepArgs& a, cudaStream_t st) {
+  return shape == 6 ? launch_potts<6>(3, a, st) : shape == 7 ? launch_potts<7>(3, a, st) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_batch_phase(int shape, int which, const BatchArgs& b, int ntiles, cudaStream_t st) {

@@ -3,7 +3,7 @@
 // delta(s_i, s_j), states 0..q-1 as int8.
 //
 // A sweep runs on the tiled path of the Ising sweep (tile shape
-// kPottsShape, 128 x 64 sites):
+// potts_shape, 128 x 64 or 128 x 32 sites):
 //   phase 1  bonds and tile clusters: an edge bonds iff its two states are
 //            equal and its word of the site pair's Philox block (C5) is
 //            below thr, thr from p = 1 - exp(-beta); then the band-scan
@@ -59,7 +59,7 @@ int pfail(int code, const char* what) { return sw::record_error(code, what); }
 }  // namespace
 
 struct sw_potts {
-  int L = 0, q = 0;
+  int L = 0, q = 0, shape = 0;
   uint32_t thr = 0;
   sw::KeySchedule ks{};
   int64_t t = 0, t_base = 0, cap = 0;
@@ -155,8 +155,8 @@ sw::SweepArgs args_of(const sw_potts* h) {
 // Phases 1-2 of the current states and counter: bonds, tile clusters, the
 // merge and each border cluster's new state.
 int clusters(sw_potts* h, const sw::SweepArgs& a) {
-  P_CUDA(sw::launch_potts_phase1(a, h->stream), "Potts phase 1 launch");
-  P_CUDA(sw::launch_phase2(sw::kPottsShape, a, h->stream), "Potts phase 2 launch");
+  P_CUDA(sw::launch_potts_phase1(h->shape, a, h->stream), "Potts phase 1 launch");
+  P_CUDA(sw::launch_phase2(h->shape, a, h->stream), "Potts phase 2 launch");
   return SW_OK;
 }
 
@@ -187,7 +187,8 @@ int sw_potts_create(int32_t L, int32_t q, double beta, uint64_t seed, int32_t in
   h->q = q;
   h->thr = potts_thr(beta);
   h->ks = sw::make_key_schedule(seed);
-  const sw::TileShape ts = sw::shape_of(sw::kPottsShape);
+  h->shape = sw::potts_shape(L);
+  const sw::TileShape ts = sw::shape_of(h->shape);
   h->g.L = L;
   h->g.tiles_x = (L + ts.tw() - 1) / ts.tw();
   h->g.tiles_y = (L + ts.th - 1) / ts.th;
@@ -243,7 +244,7 @@ int sw_potts_sweep(sw_potts* h, int32_t n) {
     a.em = h->em + 2 * (h->t - h->t_base);  // zeroed by phase 1
     rc = clusters(h, a);
     if (rc != SW_OK) return rc;
-    P_CUDA(sw::launch_potts_phase3(a, h->stream), "Potts phase 3 launch");
+    P_CUDA(sw::launch_potts_phase3(h->shape, a, h->stream), "Potts phase 3 launch");
     h->t += 1;
   }
   return SW_OK;
@@ -311,7 +312,7 @@ int sw_potts_labels(sw_potts* h, int32_t* out, int32_t out_is_device) {
   int rc = clusters(h, a);
   if (rc != SW_OK) return rc;
   a.labels = dst;
-  P_CUDA(sw::launch_phase3(sw::kPottsShape, a, true, h->stream), "labels launch");
+  P_CUDA(sw::launch_phase3(h->shape, a, true, h->stream), "labels launch");
   if (out_is_device) return SW_OK;
   P_CUDA(cudaMemcpyAsync(out, dst, n * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream), "labels copy");
   return check_potts(h);

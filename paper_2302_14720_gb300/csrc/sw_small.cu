@@ -465,9 +465,9 @@ size_t small_smem_bytes(int L) {
 }  // namespace
 
 cudaError_t launch_small(const SmallArgs& a, cudaStream_t st) {
-  if (a.L < 2 || a.L > kSmallChainMaxL) return cudaErrorInvalidValue;
+  if (a.L < 2 || a.L > kSmallMaxL) return cudaErrorInvalidValue;
   if (a.n <= 0) return cudaSuccess;
-  const size_t dyn = small_smem_bytes(kSmallChainMaxL);
+  const size_t dyn = small_smem_bytes(kSmallMaxL);
   static bool attr_done = false;  // set once per process; the attribute is per function
   if (!attr_done) {
     const cudaError_t e =
