@@ -97,6 +97,33 @@ namespace sw {
 int record_error(int code, const char* msg) { return fail(code, "%s", msg); }
 }  // namespace sw
 
+namespace sw {
+namespace {
+__global__ void read_back_kernel(const int* err, const unsigned long long* src, int words, unsigned long long* page) {
+  after_previous();
+  if (threadIdx.x == 0) page[0] = (unsigned long long)(unsigned)*err;
+  for (int i = threadIdx.x; i < words; i += blockDim.x) page[1 + i] = src[i];
+}
+}  // namespace
+
+cudaError_t ReadBack::operator()(cudaStream_t st, const int* err, const void* src, size_t words, int* flag, void* out) {
+  if (!page_) {
+    const cudaError_t e = cudaHostAlloc(&page_, kPageWords * sizeof *page_, cudaHostAllocDefault);
+    if (e != cudaSuccess) return e;
+  }
+  const bool fits = words < kPageWords;
+  cudaError_t e = launch_after(read_back_kernel, 1, words > 128 ? 512 : 128, 0, st, err,
+                               static_cast<const unsigned long long*>(src), fits ? (int)words : 0, page_);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return e;
+  *flag = (int)(unsigned)page_[0];
+  if (*flag != 0 || words == 0) return cudaSuccess;
+  if (!fits) return cudaMemcpy(out, src, words * sizeof *page_, cudaMemcpyDeviceToHost);
+  memcpy(out, page_ + 1, words * sizeof *page_);
+  return cudaSuccess;
+}
+}  // namespace sw
+
 struct sw_lattice {
   int L = 0;
   double beta = 0.0;
@@ -105,6 +132,7 @@ struct sw_lattice {
   int64_t t = 0;       // next sweep counter (absolute)
   int64_t t_base = 0;  // first sweep held in the trace
   int64_t cap = 0;     // trace capacity in sweeps
+  sw::ReadBack read;
   int shape = 0;
   int device = 0;
   bool hist_on = false;
@@ -271,11 +299,11 @@ int ensure_trace(sw_lattice* h, int64_t sweeps_needed) {
   return SW_OK;
 }
 
-// Synchronise the handle's stream and turn the device error flag into a status.
-int sync_and_check(sw_lattice* h) {
-  SW_CUDA(cudaStreamSynchronize(h->stream), "stream synchronize");
+// Synchronise the handle's stream, turn the device error flag into a status
+// and, if it is clear, read `words` words of device memory at src into out.
+int sync_and_check(sw_lattice* h, const void* src = nullptr, size_t words = 0, void* out = nullptr) {
   int flag = 0;
-  SW_CUDA(cudaMemcpy(&flag, h->tb.err, sizeof(int), cudaMemcpyDeviceToHost), "error flag read");
+  SW_CUDA(h->read(h->stream, h->tb.err, src, words, &flag, out), "stream synchronize and read");
   switch (flag) {
     case sw::kErrNone: return SW_OK;
     case sw::kErrUnionCap: return fail(SW_ETIMEOUT, "device union-find retry loop reached its cap");
@@ -474,16 +502,12 @@ int sw_observables(sw_lattice* h, int64_t first, int64_t count, int64_t* E_host,
   if (!h) return fail(SW_EINVAL, "handle is NULL");
   int rc = range_ok(h, first, count);
   if (rc != SW_OK) return rc;
-  rc = sync_and_check(h);
-  if (rc != SW_OK) return rc;
-  if (count == 0) return SW_OK;
-  int64_t* tmp = (int64_t*)malloc((size_t)count * 2 * sizeof(int64_t));
-  if (!tmp) return fail(SW_ENOMEM, "host allocation failed");
-  cudaError_t e = cudaMemcpy(tmp, h->em + 2 * (first - h->t_base), (size_t)count * 2 * sizeof(int64_t),
-                             cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) {
+  int64_t* tmp = count ? (int64_t*)malloc((size_t)count * 2 * sizeof(int64_t)) : nullptr;
+  if (count && !tmp) return fail(SW_ENOMEM, "host allocation failed");
+  rc = sync_and_check(h, h->em + 2 * (first - h->t_base), (size_t)count * 2, tmp);
+  if (rc != SW_OK) {
     free(tmp);
-    return cuda_fail(e, "trace copy");
+    return rc;
   }
   for (int64_t k = 0; k < count; ++k) {
     if (E_host) E_host[k] = tmp[2 * k];
@@ -511,13 +535,7 @@ int sw_histograms(sw_lattice* h, int64_t first, int64_t count, int64_t* out_host
   int rc = range_ok(h, first, count);
   if (rc != SW_OK) return rc;
   if (count > 0 && !out_host) return fail(SW_EINVAL, "out_host is NULL");
-  rc = sync_and_check(h);
-  if (rc != SW_OK) return rc;
-  if (count == 0) return SW_OK;
-  SW_CUDA(cudaMemcpy(out_host, h->hist + SW_HIST_WORDS * (first - h->t_base),
-                     (size_t)count * SW_HIST_WORDS * sizeof(int64_t), cudaMemcpyDeviceToHost),
-          "histogram copy");
-  return SW_OK;
+  return sync_and_check(h, h->hist + SW_HIST_WORDS * (first - h->t_base), (size_t)count * SW_HIST_WORDS, out_host);
 }
 
 int sw_labels(sw_lattice* h, int32_t* out, int32_t out_is_device) {

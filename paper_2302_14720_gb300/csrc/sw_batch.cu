@@ -63,6 +63,7 @@ struct sw_batch {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int* d_err = nullptr;
+  sw::ReadBack read;
   std::vector<Replica> reps;
   sw::ReplicaDesc* d_descs = nullptr;
   int desc_cap = 0;
@@ -257,10 +258,10 @@ int check_slot(sw_batch* b, int32_t slot) {
   return SW_OK;
 }
 
-int sync_and_check_batch(sw_batch* b) {
-  B_CUDA(cudaStreamSynchronize(b->stream), "stream synchronize");
+// As sync_and_check of a lattice.
+int sync_and_check_batch(sw_batch* b, const void* src = nullptr, size_t words = 0, void* out = nullptr) {
   int flag = 0;
-  B_CUDA(cudaMemcpy(&flag, b->d_err, sizeof(int), cudaMemcpyDeviceToHost), "error flag read");
+  B_CUDA(b->read(b->stream, b->d_err, src, words, &flag, out), "stream synchronize and read");
   if (flag == sw::kErrUnionCap) return bfail(SW_ETIMEOUT, "device union-find retry loop reached its cap");
   if (flag == sw::kErrCopyTimeout) return bfail(SW_ETIMEOUT, "device bulk copy into shared memory did not complete");
   if (flag == sw::kErrBarrierTimeout) return bfail(SW_ETIMEOUT, "a grid barrier of the fused batch kernel did not open");
@@ -515,13 +516,9 @@ int sw_batch_observables(sw_batch* b, int32_t slot, int64_t first, int64_t count
   if (rc != SW_OK) return rc;
   const Replica& r = b->reps[slot];
   if (count < 0 || first < r.t_base || first + count > r.t) return bfail(SW_EINVAL, "sweeps outside the trace");
-  rc = sync_and_check_batch(b);
-  if (rc != SW_OK) return rc;
-  if (count == 0) return SW_OK;
   std::vector<int64_t> tmp((size_t)count * 2);
-  B_CUDA(cudaMemcpy(tmp.data(), r.em + 2 * (first - r.t_base), (size_t)count * 2 * sizeof(int64_t),
-                    cudaMemcpyDeviceToHost),
-         "trace copy");
+  rc = sync_and_check_batch(b, r.em + 2 * (first - r.t_base), tmp.size(), tmp.data());
+  if (rc != SW_OK) return rc;
   for (int64_t k = 0; k < count; ++k) {
     if (E_host) E_host[k] = tmp[2 * k];
     if (M_host) M_host[k] = tmp[2 * k + 1];

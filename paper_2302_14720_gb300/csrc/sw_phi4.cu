@@ -743,6 +743,7 @@ struct sw_phi4 {
   double* obs = nullptr;  // [cap][5]: E, M0..M3
   uint32_t* top = nullptr;  // [2], by update parity: high word of the field's largest |component| (projection -> E and M)
   int* err = nullptr;
+  sw::ReadBack read;
 };
 
 namespace {
@@ -763,10 +764,10 @@ void free_phi4(sw_phi4* h) {
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
-int check_phi4(sw_phi4* h) {
-  F_CUDA(cudaStreamSynchronize(h->stream), "stream synchronize");
+// As sync_and_check of an Ising lattice.
+int check_phi4(sw_phi4* h, const void* src = nullptr, size_t words = 0, void* out = nullptr) {
   int flag = 0;
-  F_CUDA(cudaMemcpy(&flag, h->err, sizeof(int), cudaMemcpyDeviceToHost), "error flag read");
+  F_CUDA(h->read(h->stream, h->err, src, words, &flag, out), "stream synchronize and read");
   if (flag == 1) return ffail(SW_ETIMEOUT, "a capped union-find loop gave up");
   if (flag != 0) return ffail(SW_EDEVICE, "device error flag set");
   return SW_OK;
@@ -969,23 +970,16 @@ int sw_phi4_sweep(sw_phi4* h, int32_t n) {
 int sw_phi4_observables(sw_phi4* h, int64_t first, int64_t count, double* E_host, double* M_host) {
   if (!h) return ffail(SW_EINVAL, "handle is NULL");
   if (count < 0 || first < h->t_base || first + count > h->t) return ffail(SW_EINVAL, "update range outside the trace");
-  int rc = check_phi4(h);
-  if (rc != SW_OK) return rc;
-  if (count == 0) return SW_OK;
-  double* buf = (double*)malloc((size_t)count * 5 * sizeof(double));
-  if (!buf) return ffail(SW_ENOMEM, "host allocation failed");
-  cudaError_t e = cudaMemcpy(buf, h->obs + 5 * (first - h->t_base), (size_t)count * 5 * sizeof(double),
-                             cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) {
-    for (int64_t k = 0; k < count; ++k) {
-      if (E_host) E_host[k] = buf[5 * k];
-      if (M_host)
-        for (int a = 0; a < 4; ++a) M_host[4 * k + a] = buf[5 * k + 1 + a];
-    }
+  double* buf = count ? (double*)malloc((size_t)count * 5 * sizeof(double)) : nullptr;
+  if (count && !buf) return ffail(SW_ENOMEM, "host allocation failed");
+  const int rc = check_phi4(h, h->obs + 5 * (first - h->t_base), (size_t)count * 5, buf);
+  for (int64_t k = 0; rc == SW_OK && k < count; ++k) {
+    if (E_host) E_host[k] = buf[5 * k];
+    if (M_host)
+      for (int a = 0; a < 4; ++a) M_host[4 * k + a] = buf[5 * k + 1 + a];
   }
   free(buf);
-  F_CUDA(e, "trace copy");
-  return SW_OK;
+  return rc;
 }
 
 int sw_phi4_field(sw_phi4* h, double* out, int32_t out_is_device) {

@@ -67,6 +67,7 @@ struct sw_potts {
   bool own_stream = false;
   sw::Geometry g{};
   sw::TileBuffers tb{};
+  sw::ReadBack read;
   int8_t* s = nullptr;        // states [L][L]
   int8_t* staging = nullptr;  // sw_potts_set_state's checked copy
   int32_t* label_buf = nullptr;
@@ -93,11 +94,10 @@ void free_potts(sw_potts* h) {
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
-// Synchronise and turn the device error flag into a status.
-int check_potts(sw_potts* h) {
-  P_CUDA(cudaStreamSynchronize(h->stream), "stream synchronize");
+// As sync_and_check of an Ising lattice.
+int check_potts(sw_potts* h, const void* src = nullptr, size_t words = 0, void* out = nullptr) {
   int flag = 0;
-  P_CUDA(cudaMemcpy(&flag, h->tb.err, sizeof(int), cudaMemcpyDeviceToHost), "error flag read");
+  P_CUDA(h->read(h->stream, h->tb.err, src, words, &flag, out), "stream synchronize and read");
   switch (flag) {
     case sw::kErrNone: return SW_OK;
     case sw::kErrUnionCap: return pfail(SW_ETIMEOUT, "a capped union-find loop gave up");
@@ -253,22 +253,15 @@ int sw_potts_sweep(sw_potts* h, int32_t n) {
 int sw_potts_observables(sw_potts* h, int64_t first, int64_t count, int64_t* E_host, int64_t* M_host) {
   if (!h) return pfail(SW_EINVAL, "handle is NULL");
   if (count < 0 || first < h->t_base || first + count > h->t) return pfail(SW_EINVAL, "sweep range outside the trace");
-  int rc = check_potts(h);
-  if (rc != SW_OK) return rc;
-  if (count == 0) return SW_OK;
-  int64_t* buf = (int64_t*)malloc((size_t)count * 2 * sizeof(int64_t));
-  if (!buf) return pfail(SW_ENOMEM, "host allocation failed");
-  cudaError_t e = cudaMemcpy(buf, h->em + 2 * (first - h->t_base), (size_t)count * 2 * sizeof(int64_t),
-                             cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) {
-    for (int64_t k = 0; k < count; ++k) {
-      if (E_host) E_host[k] = buf[2 * k];
-      if (M_host) M_host[k] = buf[2 * k + 1];
-    }
+  int64_t* buf = count ? (int64_t*)malloc((size_t)count * 2 * sizeof(int64_t)) : nullptr;
+  if (count && !buf) return pfail(SW_ENOMEM, "host allocation failed");
+  const int rc = check_potts(h, h->em + 2 * (first - h->t_base), (size_t)count * 2, buf);
+  for (int64_t k = 0; rc == SW_OK && k < count; ++k) {
+    if (E_host) E_host[k] = buf[2 * k];
+    if (M_host) M_host[k] = buf[2 * k + 1];
   }
   free(buf);
-  P_CUDA(e, "trace copy");
-  return SW_OK;
+  return rc;
 }
 
 int sw_potts_states(sw_potts* h, int8_t* out, int32_t out_is_device) {
