@@ -486,8 +486,9 @@ int sw_shape_info(int32_t shape, int32_t* tile_w, int32_t* tile_h, int32_t* stri
 /* Process-wide preference: lattices whose side L has ceil(log2 L) ==
  * log2_bucket (0..16) use `shape` from now on in sw_create, and batches
  * created with shape -1 use the entry of their largest L; shape -1 restores
- * the built-in default (64x64 tiles up to L = 64; then for a lattice 128x32
- * tiles up to L = 1024 and 128x64 above, for a batch 128x64). Results never
+ * the built-in default (for a lattice 128x32
+ * tiles up to L = 1024 and 128x64 above, for a batch of at most 608 tiles of
+ * 128x64 sites 128x32 and 128x64 above). Results never
  * depend on the shape. */
 int sw_tune_shape(int32_t log2_bucket, int32_t shape);
 

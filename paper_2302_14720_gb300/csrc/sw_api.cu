@@ -66,7 +66,7 @@ int bucket_of(int L) {
 
 // lattice: the shape of a lone lattice (sw_create); else of a batch whose
 // largest side is L.
-int shape_for(int L, bool lattice) {
+int shape_for(int L, bool lattice, int64_t batch_tiles = 0) {
   if (const char* env = getenv("SW_TILE_SHAPE")) {
     const int v = atoi(env);
     if (v >= 0 && v < sw::kNumShapes) return v;
@@ -76,21 +76,25 @@ int shape_for(int L, bool lattice) {
   });
   const int t = g_tuned[bucket_of(L)].load();
   if (t >= 0) return t;
-  if (!lattice && L <= 64) return 2;
   // A lone lattice of side <= 1024 has at most 128 tiles of 128 x 64, less
   // than one wave of 152 SMs; with 128 x 32 tiles twice as many CTAs share
   // each phase's latency, and in phase 3 a thread has one row word (one-row
   // strips) instead of two to walk. With these strips phases 1 and 3 take the
   // same block, so that chains run them in one launch: L = 256 44.5 -> 36.7
-  // us a sweep, 1024 49.9 -> 40.3, with statistics 78 -> 64. Batches keep
-  // 128 x 64.
-  return lattice && L <= 1024 ? 7 : 6;
+  // us a sweep, 1024 49.9 -> 40.3, with statistics 78 -> 64.
+  if (lattice) return L <= 1024 ? 7 : 6;
+  // A batch by the same rule as long as its replicas have at most four 128 x
+  // 64 tiles an SM (8 replicas up to L = 64 55 -> 38 us a sweep, 128 replicas
+  // up to 256, 470 tiles, 114 -> 106), 128 x 64 tiles above (256 replicas up
+  // to 1024, 9100 tiles, 573 against 643).
+  if (batch_tiles > 0 && batch_tiles <= 4 * 152) return 7;
+  return L <= 64 ? 2 : 6;
 }
 
 }  // namespace
 
 namespace sw {
-int default_shape(int L) { return shape_for(L, false); }
+int default_shape(int L, int64_t tiles) { return shape_for(L, false, tiles); }
 }  // namespace sw
 
 namespace sw {

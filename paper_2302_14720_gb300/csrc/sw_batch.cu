@@ -60,6 +60,7 @@ void free_replica(Replica& r) {
 
 struct sw_batch {
   int shape = 0;
+  bool own_shape = false;  // the library chose the shape
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int* d_err = nullptr;
@@ -288,8 +289,13 @@ int sw_batch_create(int32_t n, const int32_t* L, const double* beta, const uint6
   if (!b) return bfail(SW_ENOMEM, "host allocation failed");
   if (shape < 0) {
     int lmax = 2;
-    for (int32_t i = 0; i < n; ++i) lmax = L[i] > lmax ? L[i] : lmax;
-    shape = sw::default_shape(lmax);
+    int64_t tiles = 0;
+    for (int32_t i = 0; i < n; ++i) {
+      lmax = L[i] > lmax ? L[i] : lmax;
+      if (L[i] >= 2) tiles += ((int64_t)L[i] + 127) / 128 * (((int64_t)L[i] + 63) / 64);
+    }
+    shape = sw::default_shape(lmax, tiles);
+    b->own_shape = true;
   }
   b->shape = shape;
   cudaError_t e = cudaSuccess;
@@ -472,7 +478,7 @@ int sw_batch_set_schedule(sw_batch* b, int32_t schedule) {
   if (!b) return bfail(SW_EINVAL, "batch is NULL");
   if (schedule != SW_SCHEDULE_PHASES && schedule != SW_SCHEDULE_FUSED)
     return bfail(SW_EINVAL, "schedule must be SW_SCHEDULE_PHASES or SW_SCHEDULE_FUSED");
-  if (schedule == SW_SCHEDULE_FUSED && !sw::batch_fused_supported(b->shape))
+  if (schedule == SW_SCHEDULE_FUSED && !sw::batch_fused_supported(b->shape, b->own_shape))
     return bfail(SW_EINVAL, "the fused schedule needs a tile shape whose phases 1 and 3 take the same block");
   if (schedule != b->schedule) {
     B_CUDA(cudaStreamSynchronize(b->stream), "stream synchronize");

@@ -184,7 +184,9 @@ int record_error(int code, const char* msg);
 
 // Tile shape for a lattice of side L: SW_TILE_SHAPE override, else the
 // tuned entry of L's size bucket, else the built-in default.
-int default_shape(int L);
+// For a batch, L is the largest side and `tiles` the 128 x 64 tiles of its
+// replicas (0: none yet).
+int default_shape(int L, int64_t tiles);
 
 // Launchers (sw_kernels.cu). Each returns cudaGetLastError() of its launches.
 cudaError_t launch_init(int8_t* spins, int L, uint64_t seed, int cold, cudaStream_t st);
@@ -203,10 +205,10 @@ cudaError_t launch_batch_phase(int shape, int which, const BatchArgs& b, int nti
 cudaError_t launch_batch_advance(const BatchArgs& b, cudaStream_t st);
 // Batch, fused schedule: one cooperative launch runs nsweeps whole sweeps of
 // every replica with tiles (all four phases, grid barriers between them) and
-// advances the replicas' counters itself. Only shapes of 64 rows and more
-// whose phases 1 and 3 take the same block (TH == 32 H) have it:
-// batch_fused_supported.
-bool batch_fused_supported(int shape);
+// advances the replicas' counters itself. Only shapes whose phases 1 and 3
+// take the same block (TH == 32 H) have it, and 128 x 32 only where the
+// library chose that shape.
+bool batch_fused_supported(int shape, bool own_shape);
 // Phase 3 of sweep t (a3) and phase 1 of sweep t + 1 (a1) in one launch, the
 // new spins handed over in shared memory (flip or assignment rule, no
 // statistics). Shapes whose phases 1 and 3 take the same block.
