@@ -553,6 +553,16 @@ __device__ __forceinline__ uint2 bond_draws(uint32_t i0, int L, uint32_t t, uint
   return make_uint2(__brev(~rE), __brev(~rS));
 }
 
+// Chains of dependent shared-memory loads that a thread follows at a time (a
+// run's label and root; a new label's ancestors). Tiles of 64 rows and more
+// come in numbers that fill the SMs, where other warps hide the latency and
+// more than one at a time costs instructions; 32-row tiles serve lattices
+// with a tile or two an SM.
+template <int TH>
+constexpr int in_step() {
+  return TH <= 32 ? 4 : 1;
+}
+
 // Phase 1 runs one warp per 32-column band and asks for 1280 resident
 // threads an SM (at most 51 registers a thread; ten CTAs of 128 threads also
 // fit their shared memory).
@@ -897,15 +907,41 @@ __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const Sweep
     for (int j = 0; j < RPL; ++j) {
       const int y = lane + 32 * j, base = y * TW + 32 * w;
       uint32_t roots = 0u;
-      for (uint32_t m = mS[j] & ~mF[j]; m; m &= m - 1) {
-        const int b = __ffs(m) - 1, x = base + b;
-        int r = par[x];
-        if (r == x) {
-          roots |= 1u << b;
-        } else {
-          r = par[par[r]];
-          for (int p = par[r]; p != r; p = par[r]) r = p;
-          par[x] = (uint16_t)r;
+      constexpr int KIN = in_step<TH>();
+      for (uint32_t m = mS[j] & ~mF[j]; m;) {
+        if (KIN == 1) {
+          const int b = __ffs(m) - 1, x = base + b;
+          m &= m - 1;
+          int r = par[x];
+          if (r == x) {
+            roots |= 1u << b;
+          } else {
+            r = par[par[r]];
+            for (int p = par[r]; p != r; p = par[r]) r = p;
+            par[x] = (uint16_t)r;
+          }
+        } else {  // KIN labels in step, the last one again past the end
+          int x[KIN], r[KIN], p[KIN];
+#pragma unroll
+          for (int i = 0; i < KIN; ++i) {
+            x[i] = m ? base + __ffs(m) - 1 : x[i - (i > 0)];
+            m &= m - 1;
+            r[i] = par[x[i]];
+          }
+#pragma unroll
+          for (int i = 0; i < KIN; ++i)
+            if (r[i] == x[i]) roots |= 1u << (x[i] - base);
+#pragma unroll
+          for (int i = 0; i < KIN; ++i) r[i] = par[r[i]];
+#pragma unroll
+          for (int i = 0; i < KIN; ++i) r[i] = par[r[i]];
+#pragma unroll
+          for (int i = 0; i < KIN; ++i) p[i] = par[r[i]];
+#pragma unroll
+          for (int i = 0; i < KIN; ++i) {
+            for (; p[i] != r[i]; p[i] = par[r[i]]) r[i] = p[i];
+            if (r[i] != x[i]) par[x[i]] = (uint16_t)r[i];
+          }
         }
       }
       rb[y * WPR + w] = roots;
@@ -914,20 +950,34 @@ __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const Sweep
   __syncthreads();
 
   // ---- border components -> slots (rank of the root in index order) and global nodes
-  for (int j0 = 0; j0 < NB; j0 += NT) {  // the same trips in every lane (a warp-wide walk)
-    const int j = j0 + tid;
-    int y = 0, x = 0, r = 0;  // a lane without a border site walks from site 0, a root
-    const bool ok = j < NB && border_site<TW, TH>(P, j, y, x);
-    if (ok) r = par[y * TW + x];
-    int p = par[r];
-    while (__any_sync(0xffffffffu, p != r)) {
-      if (p != r) {
-        r = p;
-        p = par[r];
+  constexpr int KB = TH <= 32 ? (NB + NT - 1) / NT : 1;  // border sites a lane walks in step (in_step)
+  for (int j0 = 0; j0 < NB; j0 += KB * NT) {             // the same trips in every lane (a warp-wide walk)
+    int r[KB];
+    bool ok[KB];
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      const int j = j0 + NT * i + tid;
+      int y = 0, x = 0;
+      r[i] = 0;  // a lane without a border site walks from site 0, a root
+      ok[i] = j < NB && border_site<TW, TH>(P, j, y, x);
+      if (ok[i]) r[i] = par[y * TW + x];
+    }
+    bool more = true;
+    while (__any_sync(0xffffffffu, more)) {
+      more = false;
+#pragma unroll
+      for (int i = 0; i < KB; ++i) {
+        const int p = par[r[i]];
+        more |= p != r[i];
+        r[i] = p;
       }
     }
-    if (ok) atomicOr(&s_bmask[r >> 5], 1u << (r & 31));
-    if (j < NB) s_broot[j] = ok ? (int16_t)r : (int16_t)-1;
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      const int j = j0 + NT * i + tid;
+      if (ok[i]) atomicOr(&s_bmask[r[i] >> 5], 1u << (r[i] & 31));
+      if (j < NB) s_broot[j] = ok[i] ? (int16_t)r[i] : (int16_t)-1;
+    }
   }
   __syncthreads();
   const int nsl = block_popc_prefix<RW, NT>(s_bmask, s_pre, s_wsum);
@@ -985,7 +1035,7 @@ constexpr int phase1_min_blocks() {
 }
 
 template <int WPR, int TH, int H, bool BATCH>
-__global__ void __launch_bounds__(32 * WPR, phase1_min_blocks<32 * WPR>())
+__global__ void __launch_bounds__(32 * WPR, TH <= 32 ? 768 / (32 * WPR) : phase1_min_blocks<32 * WPR>())
     phase1_kernel(const SweepArgs a0, const BatchArgs bat) {
   if (!BATCH) after_previous();
   __shared__ P1Shared<WPR, TH, H> S;
@@ -1256,13 +1306,47 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
       for (int q = 0; q < 4; ++q) z[q] = make_int4(0, 0, 0, 0);
     }
   }
+  // the slots of the halo's sites in the neighbour tiles, and their old spins
+  const uint32_t* bbits = a.tb.bbits + (size_t)P.tile * BBW;
+  constexpr int NE = LABELS ? 0 : (TH + NT - 1) / NT, NSO = LABELS ? 0 : (TW + NT - 1) / NT;
+  uint16_t slotE[NE + 1], slotS[NSO + 1];
+  const int tileE = P.ty * g.tiles_x + (P.tx + 1) % g.tiles_x, tileS = ((P.ty + 1) % g.tiles_y) * g.tiles_x + P.tx;
+  uint32_t oldE[NE + 1], oldS[NSO + 1];
+#pragma unroll
+  for (int i = 0; i < NE; ++i) {
+    slotE[i] = tid + NT * i < P.nrows ? __ldcg(a.tb.bslot + (size_t)tileE * NB + tid + NT * i) : 0;
+    oldE[i] = warp0 + NT * i < TH ? bbits[Tl::OFF_HE + ((warp0 + NT * i) >> 5)] : 0u;
+  }
+#pragma unroll
+  for (int i = 0; i < NSO; ++i) {
+    slotS[i] = tid + NT * i < P.ncols ? __ldcg(a.tb.bslot + (size_t)tileS * NB + 2 * TH + tid + NT * i) : 0;
+    oldS[i] = warp0 + NT * i < TW ? bbits[Tl::OFF_HS + ((warp0 + NT * i) >> 5)] : 0u;
+  }
   if (HIST)
     for (int i = tid; i < 34; i += NT) s_hist[i] = 0ull;
   for (int i = tid; i < (MS + 31) / 32; i += NT) s_slotdec[i] = 0u;
   __syncthreads();
   if (block_popc_prefix<RW, NT>(s_bmask, s_pre, s_wsum) != nsl && tid == 0) atomicCAS(a.tb.err, 0, kErrSlotOverflow);
 
-  // ---- this tile's slots: root key and flip, as the resolve pass left them
+  // ---- this tile's slots: root key and flip, as the resolve pass left them;
+  // the halo's nodes (their slots came with the first loads) go out with them
+  uint64_t nodeE[NE + 1], nodeS[NSO + 1];
+#pragma unroll
+  for (int i = 0; i < NE; ++i) {
+    if (slotE[i] >= MS) {
+      atomicCAS(a.tb.err, 0, kErrSlotOverflow);
+      slotE[i] = 0;
+    }
+    nodeE[i] = tid + NT * i < P.nrows ? ld_node(a.tb.nodes + (uint32_t)tileE * MS + slotE[i]) : 0ull;
+  }
+#pragma unroll
+  for (int i = 0; i < NSO; ++i) {
+    if (slotS[i] >= MS) {
+      atomicCAS(a.tb.err, 0, kErrSlotOverflow);
+      slotS[i] = 0;
+    }
+    nodeS[i] = tid + NT * i < P.ncols ? ld_node(a.tb.nodes + (uint32_t)tileS * MS + slotS[i]) : 0ull;
+  }
   for (int j = tid; j < nsl; j += NT) {
     const uint64_t v = ld_node(a.tb.nodes + (uint32_t)P.tile * MS + j);
     if (LABELS) s_slotkey[j] = (int)((uint32_t)(v >> 32) & 0x7fffffffu);
@@ -1270,42 +1354,28 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
     if (HIST) s_slotroot[j] = (uint32_t)v;
   }
   if (!LABELS) {
-    // ---- new spins of the halo sites: old spin (phase 1) xor their cluster's
-    // flip; the two dependent loads (slot, then node) overlap the labels copy
-    const uint32_t* bbits = a.tb.bbits + (size_t)P.tile * BBW;
-    for (int b0 = warp0; b0 < TH; b0 += NT) {
-      const int y = b0 + lane;
-      bool bit = false;
-      if (y < P.nrows) {
-        const int tileE = P.ty * g.tiles_x + (P.tx + 1) % g.tiles_x;
-        uint16_t slot = __ldcg(a.tb.bslot + (size_t)tileE * NB + y);
-        if (slot >= MS) {
-          atomicCAS(a.tb.err, 0, kErrSlotOverflow);
-          slot = 0;
-        }
-        const uint64_t v = ld_node(a.tb.nodes + (uint32_t)tileE * MS + slot);
-        const uint32_t old = (bbits[Tl::OFF_HE + (y >> 5)] >> (y & 31)) & 1u;
-        bit = ((a.rule ? 0u : old) ^ (uint32_t)(v >> 63)) != 0u;
+    // ---- new spins of the halo sites: old spin (phase 1) xor their cluster's flip
+#pragma unroll
+    for (int i = 0; i < NE; ++i) {
+      const int b0 = warp0 + NT * i;
+      if (b0 >= TH) break;  // the same in every lane of the warp
+      const uint32_t m = __ballot_sync(0xffffffffu, (nodeE[i] >> 63) != 0u);
+      if (lane == 0) {
+        const int nr = max(0, min(32, P.nrows - b0));
+        const uint32_t valid = nr ? 0xffffffffu >> (32 - nr) : 0u;
+        s_hEnew[b0 >> 5] = ((a.rule ? 0u : oldE[i]) ^ m) & valid;
       }
-      const uint32_t m = __ballot_sync(0xffffffffu, bit);
-      if (lane == 0) s_hEnew[b0 >> 5] = m;
     }
-    for (int b0 = warp0; b0 < TW; b0 += NT) {
-      const int x = b0 + lane;
-      bool bit = false;
-      if (x < P.ncols) {
-        const int tileS = ((P.ty + 1) % g.tiles_y) * g.tiles_x + P.tx;
-        uint16_t slot = __ldcg(a.tb.bslot + (size_t)tileS * NB + 2 * TH + x);
-        if (slot >= MS) {
-          atomicCAS(a.tb.err, 0, kErrSlotOverflow);
-          slot = 0;
-        }
-        const uint64_t v = ld_node(a.tb.nodes + (uint32_t)tileS * MS + slot);
-        const uint32_t old = (bbits[Tl::OFF_HS + (x >> 5)] >> (x & 31)) & 1u;
-        bit = ((a.rule ? 0u : old) ^ (uint32_t)(v >> 63)) != 0u;
+#pragma unroll
+    for (int i = 0; i < NSO; ++i) {
+      const int b0 = warp0 + NT * i;
+      if (b0 >= TW) break;
+      const uint32_t m = __ballot_sync(0xffffffffu, (nodeS[i] >> 63) != 0u);
+      if (lane == 0) {
+        const int nc = max(0, min(32, P.ncols - b0));
+        const uint32_t valid = nc ? 0xffffffffu >> (32 - nc) : 0u;
+        s_hSnew[b0 >> 5] = ((a.rule ? 0u : oldS[i]) ^ m) & valid;
       }
-      const uint32_t m = __ballot_sync(0xffffffffu, bit);
-      if (lane == 0) s_hSnew[b0 >> 5] = m;
     }
   }
   __syncthreads();
@@ -1336,12 +1406,16 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
       const int y = y0r + r, base = y * TW + 32 * w, rw = y * WPR + w;
       const uint32_t bm = s_bmask[rw];
       uint32_t inner = r < nv ? rbw[r] & ~bm : 0u;
+      // the word's border roots have consecutive slots from s_pre[rw] on:
+      // their decisions are one stretch of s_slotdec's bits (clear past nsl),
+      // dealt out to the roots' columns
       uint32_t fl = 0, B = r < nv ? bm : 0u;
-      while (B) {
-        const int b = __ffs(B) - 1;
-        B &= B - 1;
-        const int sl = slot_of(s_bmask, s_pre, base + b);
-        fl |= (sl < nsl ? (s_slotdec[sl >> 5] >> (sl & 31)) & 1u : 0u) << b;
+      if (B) {
+        constexpr int DWORDS = (MS + 31) / 32;
+        const int sl = (int)s_pre[rw], q = min(sl >> 5, DWORDS - 1);
+        uint32_t dec = __funnelshift_r(s_slotdec[q], q + 1 < DWORDS ? s_slotdec[q + 1] : 0u, sl & 31);
+        for (; B; B &= B - 1, dec >>= 1)
+          if (dec & 1u) fl |= B & (0u - B);
       }
       if (!a.rule && inner) {
         fl |= flip_bits32((uint32_t)(P.y0 + y) * (uint32_t)L + (uint32_t)(P.x0 + 32 * w), a.t, a.ks) & inner;
@@ -1429,6 +1503,7 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
   // rows of whole 16-byte aligned words are stored by the threads that own
   // them, others by the block together once all words are known
   const bool vecrows = g.aligned16 && (P.ncols & 31) == 0;
+  constexpr int KIN = in_step<TH>();
   // HIST: a lane adds up the lengths of consecutive runs of one root and
   // sends the sum when the root changes (a tile's runs mostly belong to few
   // clusters near order, which made per-run shared atomics serialise)
@@ -1445,11 +1520,24 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
       uint32_t Rr = __funnelshift_r(Rall, Rall, rot);  // bit i: run start at column (i + rot) mod 32
       uint32_t D = 0u;                                // decision of each run, at its start
       while (Rr) {
-        const int b = (__ffs(Rr) - 1 + rot) & 31;
-        Rr &= Rr - 1;
-        const int rt = par[par[base + b]];  // the run's label, then the label's root
-        D |= ((s_flip[rt >> 5] >> (rt & 31)) & 1u) << b;
-        if (HIST) {
+        int bs[KIN], rts[KIN];  // the next KIN runs, the last one again past the end
+        bool have[KIN];
+#pragma unroll
+        for (int i = 0; i < KIN; ++i) {
+          have[i] = i == 0 || Rr != 0u;
+          bs[i] = have[i] ? (__ffs(Rr) - 1 + rot) & 31 : bs[i - (i > 0)];
+          Rr &= Rr - 1;  // (0 stays 0)
+        }
+#pragma unroll
+        for (int i = 0; i < KIN; ++i) rts[i] = par[base + bs[i]];  // the run's label
+#pragma unroll
+        for (int i = 0; i < KIN; ++i) rts[i] = par[rts[i]];  // the label's root
+#pragma unroll
+        for (int i = 0; i < KIN; ++i) D |= ((s_flip[rts[i] >> 5] >> (rts[i] & 31)) & 1u) << bs[i];
+#pragma unroll
+        for (int i = 0; HIST && i < KIN; ++i) {
+          if (!have[i]) continue;
+          const int b = bs[i], rt = rts[i];
           const uint32_t above = Rall & ~((2u << b) - 1u);  // run starts after b (b = 31: none)
           const uint32_t len = (uint32_t)((above ? __ffs(above) - 1 : nb) - b);
           if (rt == acc_rt) {
@@ -1738,7 +1826,7 @@ __global__ void __launch_bounds__(32 * WPR, band_min_blocks<32 * WPR>())
 // still reads this tile's tables of sweep t while this CTA writes those of
 // sweep t + 1. Every other table a tile writes is read by that tile alone.
 template <int WPR, int TH, int H>
-__global__ void __launch_bounds__(32 * WPR, band_min_blocks<32 * WPR>())
+__global__ void __launch_bounds__(32 * WPR, TH <= 32 ? 768 / (32 * WPR) : band_min_blocks<32 * WPR>())
     phase31_kernel(const SweepArgs a3, const SweepArgs a1) {
   after_previous();
   using Tl = Tile<WPR, TH, H>;
