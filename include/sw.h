@@ -130,8 +130,8 @@ int sw_destroy(sw_lattice* h);
  * sweep E and M (C10), and the C11 statistics if enabled, are appended to
  * the device-side trace. Errors: SW_EINVAL (n < 0), SW_ENOMEM (trace
  * growth), SW_ECUDA. Device-side failures are reported by the next call that
- * synchronises. A lattice with L <= 160 (144 for n = 1) and statistics off runs all n
- * sweeps in one CTA-sized launch (the whole lattice in shared memory)
+ * synchronises. A lattice with L <= 160 (144 for n = 1) and statistics off
+ * runs all n sweeps in one CTA-sized launch (the whole lattice in shared memory)
  * unless the environment variable SW_TILE_SHAPE was set at sw_create, which
  * keeps it on the tiled path; the results are the same. Between the sweeps
  * of one call the bond draws of the next sweep (C5: they depend on the
@@ -486,10 +486,10 @@ int sw_shape_info(int32_t shape, int32_t* tile_w, int32_t* tile_h, int32_t* stri
 /* Process-wide preference: lattices whose side L has ceil(log2 L) ==
  * log2_bucket (0..16) use `shape` from now on in sw_create, and batches
  * created with shape -1 use the entry of their largest L; shape -1 restores
- * the built-in default (for a lattice 128x32
- * tiles up to L = 1024 and 128x64 above, for a batch of at most 608 tiles of
- * 128x64 sites 128x32 and 128x64 above). Results never
- * depend on the shape. */
+ * the built-in default (for a lattice 128x32 tiles up to L = 1024 and 128x64
+ * above, for a batch of at most 608 tiles of 128x64 sites 128x32 and 128x64
+ * above, 64x64 if all sides are at most 64). Results never depend on the
+ * shape. */
 int sw_tune_shape(int32_t log2_bucket, int32_t shape);
 
 /* The tile shape index a lattice was created with (its tiled path; sides up

@@ -7,8 +7,8 @@ namespace sw {
 
 // ------------------------------------------------- row masks of the band scan
 //
-// Phase 1 of the tiled path, and the one-CTA path, label sites by a Hoshen-Kopelman scan down each 32-column band:
-// the rows are visited top to bottom, every run (a maximal stretch of east
+// Phase 1 of the tiled path, and the one-CTA path, label sites by a
+// Hoshen-Kopelman scan down each 32-column band: the rows are visited top to bottom, every run (a maximal stretch of east
 // bonds inside one row word) takes the label of the run above it that it is
 // bonded to, or a new label (its first site) when it has no bond upwards,
 // and a run bonded to several runs above that carry different labels makes

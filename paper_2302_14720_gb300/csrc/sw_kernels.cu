@@ -553,14 +553,19 @@ __device__ __forceinline__ uint2 bond_draws(uint32_t i0, int L, uint32_t t, uint
   return make_uint2(__brev(~rE), __brev(~rS));
 }
 
-// Chains of dependent shared-memory loads that a thread follows at a time (a
-// run's label and root; a new label's ancestors). Tiles of 64 rows and more
-// come in numbers that fill the SMs, where other warps hide the latency and
-// more than one at a time costs instructions; 32-row tiles serve lattices
-// with a tile or two an SM.
+// Chains of dependent shared-memory loads that a thread follows at a time: a
+// new label's ancestors in phase 1, a run's label and root in phase 3. 32-row
+// tiles serve lattices with a tile or two an SM, where nothing else hides the
+// latency. 64-row tiles fill the SMs: phase 1, bound by instruction issue, is
+// slower with two (250 -> 258 us at L = 8192), phase 3, bound by latency all
+// the same, faster (83.9 -> 79.9).
 template <int TH>
-constexpr int in_step() {
+constexpr int labels_in_step() {
   return TH <= 32 ? 4 : 1;
+}
+template <int TH>
+constexpr int runs_in_step() {
+  return TH <= 32 ? 4 : 2;
 }
 
 // Phase 1 runs one warp per 32-column band and asks for 1280 resident
@@ -907,7 +912,7 @@ __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const Sweep
     for (int j = 0; j < RPL; ++j) {
       const int y = lane + 32 * j, base = y * TW + 32 * w;
       uint32_t roots = 0u;
-      constexpr int KIN = in_step<TH>();
+      constexpr int KIN = labels_in_step<TH>();
       for (uint32_t m = mS[j] & ~mF[j]; m;) {
         if (KIN == 1) {
           const int b = __ffs(m) - 1, x = base + b;
@@ -950,7 +955,7 @@ __device__ __forceinline__ void phase1_body(P1Shared<WPR, TH, H>& S, const Sweep
   __syncthreads();
 
   // ---- border components -> slots (rank of the root in index order) and global nodes
-  constexpr int KB = TH <= 32 ? (NB + NT - 1) / NT : 1;  // border sites a lane walks in step (in_step)
+  constexpr int KB = TH <= 32 ? (NB + NT - 1) / NT : 1;  // border sites a lane walks in step
   for (int j0 = 0; j0 < NB; j0 += KB * NT) {             // the same trips in every lane (a warp-wide walk)
     int r[KB];
     bool ok[KB];
@@ -1143,7 +1148,8 @@ constexpr int phase2_threads() {
   return TH + TW + 32 * kDrawWarps;
 }
 template <int WPR, int TH, int H, bool BATCH>
-__global__ void __launch_bounds__(phase2_threads<TH, 32 * WPR>(), 2048 / phase2_threads<TH, 32 * WPR>()) phase2_kernel(const SweepArgs a0, const BatchArgs bat) {
+__global__ void __launch_bounds__(phase2_threads<TH, 32 * WPR>(), 2048 / phase2_threads<TH, 32 * WPR>())
+    phase2_kernel(const SweepArgs a0, const BatchArgs bat) {
   if (!BATCH && !a0.draws_out) start_next();  // else when the draws are done: they are the longer part
   if (!BATCH) after_previous();
   using Tl = Tile<WPR, TH, H>;
@@ -1503,7 +1509,7 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
   // rows of whole 16-byte aligned words are stored by the threads that own
   // them, others by the block together once all words are known
   const bool vecrows = g.aligned16 && (P.ncols & 31) == 0;
-  constexpr int KIN = in_step<TH>();
+  constexpr int KIN = runs_in_step<TH>();
   // HIST: a lane adds up the lengths of consecutive runs of one root and
   // sends the sum when the root changes (a tile's runs mostly belong to few
   // clusters near order, which made per-run shared atomics serialise)
@@ -2145,8 +2151,8 @@ cudaError_t launch_all(int which, const SweepArgs& a, int mode, uint8_t* out, cu
         const size_t dyn = (size_t)TH * T::TW * sizeof(uint16_t);
         static bool attr_done = false;
         if (!attr_done) {
-          e = cudaFuncSetAttribute(phase3_kernel<WPR, TH, H, 1, false>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+          e = cudaFuncSetAttribute(phase3_kernel<WPR, TH, H, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)dyn);
           if (e != cudaSuccess) return e;
           attr_done = true;
         }
