@@ -221,8 +221,8 @@ int sw_bonds(sw_lattice* h, uint8_t* out_host);
  * 0 = bonds + tile-local clusters, 1 = cross-tile merge, 2 = flips + E/M,
  * 3 = cluster statistics, 4 = flips + E/M of a sweep together with the bonds
  * and tile-local clusters of the next sweep of the same call (one launch,
- * on the 128x32, 128x64 and 128x128 tile shapes with statistics off; a call's last
- * sweep runs phase 2 alone). Not part of the paper: measurement support. */
+ * on the 128x32, 128x64 and 128x128 tile shapes with statistics off; a
+ * call's last sweep runs phase 2 alone). Not part of the paper: measurement support. */
 #define SW_TIMING_PHASES 5
 int sw_timing(sw_lattice* h, int32_t enable);
 

@@ -8,14 +8,14 @@ namespace sw {
 // ------------------------------------------------- row masks of the band scan
 //
 // Phase 1 of the tiled path, and the one-CTA path, label sites by a
-// Hoshen-Kopelman scan down each 32-column band: the rows are visited top to bottom, every run (a maximal stretch of east
-// bonds inside one row word) takes the label of the run above it that it is
-// bonded to, or a new label (its first site) when it has no bond upwards,
-// and a run bonded to several runs above that carry different labels makes
-// those labels equivalent (a union). What each run of a row needs -- which of
-// its columns passes the label down, which columns join a further run above
-// -- follows from four bit masks of the row, computed for all runs of a word
-// at once.
+// Hoshen-Kopelman scan down each 32-column band: the rows are visited top to
+// bottom, every run (a maximal stretch of east bonds inside one row word)
+// takes the label of the run above it that it is bonded to, or a new label
+// (its first site) when it has no bond upwards, and a run bonded to several
+// runs above that carry different labels makes those labels equivalent (a
+// union). What each run of a row needs -- which of its columns passes the
+// label down, which columns join a further run above -- follows from four bit
+// masks of the row, computed for all runs of a word at once.
 
 // Bits j of D whose interval (previous bit of D below j, j] holds a bit of X
 // (for the lowest bit of D the interval starts at bit 0). One addition scans
