@@ -529,17 +529,22 @@ struct Fix4 {
   int64_t v[4];
 };
 
-// d 2^(54-T) rounded to an integer; shift0 = T + 1031. A double is m 2^(e - 1086)
-// with m its mantissa from bit 63 down, so the result is m >> (T + 1032 - e),
-// taken with one more bit, given its sign and rounded.
+// d 2^(54-T) rounded to the nearest integer, ties to even; shift0 = T + 1031.
+// A double is m 2^(e - 1086) with m its mantissa from bit 63 down, so the
+// result is m >> (T + 1032 - e), taken with one more bit and a sticky bit.
+// Components just below the bound lose a bit or two, so exact ties are common
+// and a fixed direction for them is a bias that grows with the sites (M off by
+// 1e-14 of a component at L = 36, 1e-15 so; 950 -> 1005 us an update at L = 64).
 __device__ __forceinline__ int64_t to_fixed(double d, int shift0) {
   const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
   const uint64_t m = ((uint64_t)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
   const uint32_t sh = (uint32_t)(shift0 - (int)((hi >> 20) & 0x7ffu));
-  uint64_t x;
+  uint64_t x, back;
   asm("shr.b64 %0, %1, %2;" : "=l"(x) : "l"(m), "r"(sh));  // shifts past 63 give 0
-  const int s = (int32_t)hi >> 31;
-  return (((int64_t)x ^ s) + (1 - s)) >> 1;
+  asm("shl.b64 %0, %1, %2;" : "=l"(back) : "l"(x), "r"(sh));
+  const uint32_t up = back != m ? 1u : (uint32_t)(x >> 1) & 1u;
+  const int64_t s = (int32_t)hi >> 31;
+  return ((int64_t)((x + up) >> 1) ^ s) - s;
 }
 __device__ __forceinline__ Fix4 to_fixed(const F4& f, int shift0) {
   return Fix4{{to_fixed(f.x, shift0), to_fixed(f.y, shift0), to_fixed(f.z, shift0), to_fixed(f.w, shift0)}};
