@@ -273,7 +273,12 @@ __global__ void __launch_bounds__(NT)
   sw::start_next();
   sw::after_previous();
   constexpr int V = B0 * B1 * B2 * B3, S1 = B0, S2 = B0 * B1, S3 = B0 * B1 * B2;
-  __shared__ float s_af[V];
+  // a warp's list of unions: a round over 32 sites may append one entry per
+  // site and direction, 96, so no list is shorter and none is left longer
+  // than CAP - 96 between rounds
+  constexpr int kRound = 3 * 32, NW = NT / 32, CAP = 2 * V / NW > kRound ? 2 * V / NW : kRound;
+  __shared__ __align__(4) uint8_t s_buf[NW * CAP * 2 > 4 * V ? NW * CAP * 2 : 4 * V];
+  float* const s_af = reinterpret_cast<float*>(s_buf);  // [V] projections, then the warps' lists
   __shared__ int s_par[V];
   __shared__ uint8_t s_b[V];  // bits 0-3: bonds inside the brick, 4-7: bonds that leave it
   const float k4f = __double2float_rn(k4);
@@ -330,11 +335,11 @@ __global__ void __launch_bounds__(NT)
   }
   __syncthreads();
   {
-    // the warp's bonds to unite, as l + V (mu - 1), listed where the
-    // projections were (V / (NT / 32) words of two entries a warp)
-    constexpr int CAP = 2 * V / (NT / 32), J = V / NT;
-    static_assert(V % NT == 0 && 3 * V <= 65536 && CAP >= 2 * 32 * J, "list entries");
-    uint16_t* const list = reinterpret_cast<uint16_t*>(s_af) + (threadIdx.x >> 5) * CAP;
+    // the warp's bonds to unite, as l + V (mu - 1)
+    constexpr int J = V / NT;
+    static_assert(V % NT == 0 && 3 * V <= 65536, "list entries");
+    static_assert(CAP >= kRound && NW * CAP * sizeof(uint16_t) <= sizeof s_buf, "a round's entries fit the list");
+    uint16_t* const list = reinterpret_cast<uint16_t*>(s_buf) + (threadIdx.x >> 5) * CAP;
     const int lane = threadIdx.x & 31;
     int n = 0;
     auto drain = [&] {
@@ -362,7 +367,7 @@ __global__ void __launch_bounds__(NT)
         if (need) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(l + V * (mu - 1));
         n += __popc(m);
       }
-      if (n > CAP - 96) drain();
+      if (n > CAP - kRound) drain();
     }
     if (n) drain();
   }
