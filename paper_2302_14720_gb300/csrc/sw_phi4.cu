@@ -518,29 +518,38 @@ __global__ void phi4_reflect_kernel(F4* phi, const double* a, const int* par, in
 // E and M of the new field. GB300's binary64 rate is about 1/60 of its
 // integer rate, and E takes 24 binary64 operations a site: at L = 64 the
 // binary64 kernel below ran 739 us, all of it in that pipe; the fixed-point one
-// runs 223 us (16.8M sites, 0.54 GB of field), bound by instruction issue.
-// Large lattices therefore sum in 64-bit fixed point: with 2^T above every |phi| (T from the
-// largest component, which the projection kernel leaves in *top; a reflection
-// keeps the length of phi), a component c becomes the integer nearest to
-// c 2^(54-T) -- exact for components down to 2^-2 of the bound, else rounded by
-// at most 2^-55 of it -- and from there on everything is exact: neighbour sums
-// and M are integer sums, and phi . S (S the sum of the four forward
-// neighbours) is taken from 27-bit low and signed high parts, each of the
-// partial products in a 64-bit sum of its own. |phi| < 2^54 and |S| < 2^56 in
-// these units, so by Cauchy-Schwarz a site adds less than 2^56 to the high
-// products, 2^58 to the mixed and 2^56 to the low ones, and sixteen sites fit.
+// runs about 265 us (16.8M sites, 0.54 GB of field), bound by instruction
+// issue: 223 us on a grid of 54 bits that every block took unchecked, and 44 us
+// for the wider grid, the check and the ordered sum of the blocks (an update
+// 1010 -> 1054 us).
+// Large lattices therefore sum in 64-bit fixed point: with 2^T above every
+// |phi| (T from the largest component, which the projection kernel leaves in
+// *top; a reflection keeps the length of phi), a component c becomes the
+// integer nearest to c 2^(58-T): exact for components down to 2^-5 of 2^T,
+// else off by at most half a unit. From there on neighbour sums, M and the
+// products phi . S (S the sum of the four forward neighbours) are integers:
+// the products from 30-bit low and signed high parts, a site's rounded once to
+// a multiple of 2^60 (2^-56 of 2^2T). |phi| <= 2^58 and |S| <= 2^60 in these
+// units, so a site adds at most 2^58 to the sum of phi . S 2^-60, its mixed
+// products stay below 2^62.4 and the low ones below 2^62, and sixteen sites fit.
+//
+// One grid for the whole field serves fields whose components lie within a few
+// orders of magnitude. Each block checks that on its own sites (kMeanBits,
+// kProductBits) and takes binary64 sums where it does not hold: a few large
+// sites among ordinary ones, a component that is small everywhere, large and
+// tiny sites in turn.
 
 struct Fix4 {
   int64_t v[4];
 };
 
-// d 2^(54-T) rounded to the nearest integer, ties to even; shift0 = T + 1031.
+// d 2^(58-T) rounded to the nearest integer, ties to even; shift0 = T + 1027.
 // A double is m 2^(e - 1086) with m its mantissa from bit 63 down, so the
-// result is m >> (T + 1032 - e), taken with one more bit and a sticky bit.
-// Components just below the bound lose a bit or two, so exact ties are common
-// and a fixed direction for them is a bias that grows with the sites (M off by
-// 1e-14 of a component at L = 36, 1e-15 so; 950 -> 1005 us an update at L = 64).
-__device__ __forceinline__ int64_t to_fixed(double d, int shift0) {
+// result is m >> (T + 1028 - e), taken with one more bit and a sticky bit.
+// (Components just below the exact range lose a bit or two, so exact ties are
+// common and a fixed direction for them would be a bias that grows with the
+// sites.) lost: a bit of d fell off the grid.
+__device__ __forceinline__ int64_t to_fixed(double d, int shift0, bool& lost) {
   const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
   const uint64_t m = ((uint64_t)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
   const uint32_t sh = (uint32_t)(shift0 - (int)((hi >> 20) & 0x7ffu));
@@ -548,18 +557,29 @@ __device__ __forceinline__ int64_t to_fixed(double d, int shift0) {
   asm("shr.b64 %0, %1, %2;" : "=l"(x) : "l"(m), "r"(sh));  // shifts past 63 give 0
   asm("shl.b64 %0, %1, %2;" : "=l"(back) : "l"(x), "r"(sh));
   const uint32_t up = back != m ? 1u : (uint32_t)(x >> 1) & 1u;
+  lost = (back != m || (x & 1u)) && ((hi << 1) | lo) != 0u;  // (a zero has no leading bit to lose)
   const int64_t s = (int32_t)hi >> 31;
   return ((int64_t)((x + up) >> 1) ^ s) - s;
 }
 __device__ __forceinline__ Fix4 to_fixed(const F4& f, int shift0) {
-  return Fix4{{to_fixed(f.x, shift0), to_fixed(f.y, shift0), to_fixed(f.z, shift0), to_fixed(f.w, shift0)}};
+  bool lost;
+  return Fix4{{to_fixed(f.x, shift0, lost), to_fixed(f.y, shift0, lost), to_fixed(f.z, shift0, lost),
+               to_fixed(f.w, shift0, lost)}};
+}
+// The same, with the components that lost bits counted in the bytes of `lost`.
+__device__ __forceinline__ Fix4 to_fixed(const F4& f, int shift0, uint32_t& lost) {
+  bool l0, l1, l2, l3;
+  const Fix4 r{{to_fixed(f.x, shift0, l0), to_fixed(f.y, shift0, l1), to_fixed(f.z, shift0, l2),
+                to_fixed(f.w, shift0, l3)}};
+  lost = (l0 ? 1u : 0u) | (l1 ? 1u << 8 : 0u) | (l2 ? 1u << 16 : 0u) | (l3 ? 1u << 24 : 0u);
+  return r;
 }
 
-// Adds the block's sums of v[0..4] to out[0..4]. The five values are reduced
+// The block's sums of v[0..4], in threads 0..4. The five values are reduced
 // together: two of them share each of the first three exchange steps (a lane
 // keeps one and passes the other on), so a warp takes 8 binary64 additions
 // instead of 25 (this pipe bounds the kernels that end here).
-__device__ __forceinline__ void block_add5(const double v[5], double* out) {
+__device__ __forceinline__ double block_sum5(const double v[5]) {
   __shared__ double red[5][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   auto pass = [&](double keep0, double keep1, int bit) {  // lanes with the bit keep the second value
@@ -573,38 +593,65 @@ __device__ __forceinline__ void block_add5(const double v[5], double* out) {
   w += __shfl_xor_sync(0xffffffffu, w, 16);
   if (lane < 5) red[lane][warp] = w;
   __syncthreads();
-  if (threadIdx.x < 5) {
-    double s = 0.0;
+  double s = 0.0;
+  if (threadIdx.x < 5)
     for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += red[threadIdx.x][k];
-    atomicAdd(out + threadIdx.x, s);
-  }
+  return s;
 }
 
-// Binary64 sums of the sites x0, x0 + step, ... below n.
-__device__ void observe_binary64(const F4* phi, int L, int64_t n, int64_t x0, int64_t step, double v[5]) {
-  for (int64_t i = x0; i < n; i += step) {
-    const uint32_t x = (uint32_t)i;
-    const Coords k = coords_of(x, (uint32_t)L);
-    const F4 f = phi[x];
-    uint32_t stride = 1;
-    for (int mu = 0; mu < 4; ++mu) {
-      const F4 g = phi[nb(x, mu, k, (uint32_t)L, stride)];
-      v[0] += f.x * g.x + f.y * g.y + f.z * g.z + f.w * g.w;
-      stride *= (uint32_t)L;
-    }
-    v[1] += f.x;
-    v[2] += f.y;
-    v[3] += f.z;
-    v[4] += f.w;
+// Adds site x's terms to the binary64 sums v.
+__device__ __forceinline__ void observe_site(const F4* phi, uint32_t L, uint32_t x, double v[5]) {
+  const Coords k = coords_of(x, L);
+  const F4 f = phi[x];
+  uint32_t stride = 1;
+  for (int mu = 0; mu < 4; ++mu) {
+    const F4 g = phi[nb(x, mu, k, L, stride)];
+    v[0] += f.x * g.x + f.y * g.y + f.z * g.z + f.w * g.w;
+    stride *= L;
   }
+  v[1] += f.x;
+  v[2] += f.y;
+  v[3] += f.z;
+  v[4] += f.w;
 }
 
 __global__ void phi4_observe_kernel(const F4* phi, int L, int64_t n, double* out /* E, M0..M3 */) {
   sw::start_next();
   sw::after_previous();
   double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  observe_binary64(phi, L, n, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, v);
-  block_add5(v, out);
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
+    observe_site(phi, (uint32_t)L, (uint32_t)x, v);
+  const double s = block_sum5(v);
+  if (threadIdx.x < 5) atomicAdd(out + threadIdx.x, s);
+}
+
+// The grid's sums of v[0..4] into out[0..4]: every block leaves its own in
+// part[block][5], and the one that finds it is the last (*done counts them,
+// and is 0 again afterwards) adds them up in a fixed order, the same in every
+// run. With an addition into out for each of the 4096 blocks of L = 64 that sum
+// rounded as often: E and M were 1.3e-15 to 2.6e-15 off there (rms of nine
+// fields; the binary64 sums of 2432 blocks 0.8e-15 to 1.8e-15), 1.0e-16 to
+// 1.3e-16 so.
+__device__ __forceinline__ void grid_sum5(double v[5], double* part, uint32_t* done, double* out) {
+  __shared__ bool s_last;
+  const uint32_t b = blockIdx.y * gridDim.x + blockIdx.x, nb = gridDim.x * gridDim.y;
+  double s = block_sum5(v);
+  if (threadIdx.x < 5) __stcg(part + (size_t)5 * b + threadIdx.x, s);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == nb - 1u;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+#pragma unroll
+  for (int c = 0; c < 5; ++c) v[c] = 0.0;
+#pragma unroll 2
+  for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x)
+#pragma unroll
+    for (int c = 0; c < 5; ++c) v[c] += __ldcg(part + (size_t)5 * i + c);
+  s = block_sum5(v);  // (the barriers above lie between its two uses)
+  if (threadIdx.x < 5) out[threadIdx.x] = s;
+  if (threadIdx.x == 0) *done = 0u;
 }
 
 // A block takes kObserveThreads consecutive sites of the (x0, x1, x2) volume
@@ -615,6 +662,17 @@ __global__ void phi4_observe_kernel(const F4* phi, int L, int64_t n, double* out
 // are loaded and converted again: 2.25 conversions a site at L = 64.
 constexpr int kObserveThreads = 256;
 constexpr int kObserveSteps = 16;
+// What a block's sites must show for its fixed-point sums to stand, in units
+// of the grid (2^58 and 2^56 are 2^T and 2^2T there):
+//   M_c  sum |phi_c| >= 2^kMeanBits for every component c that lost bits: the
+//        half units lost add up to at most 2^-53 of that sum, half an ulp;
+//   E    sum |phi . S| >= 2^kProductBits for every site, 2^-8 of the bound. A
+//        site's phi . S is off by about 2^-59 of the bound, at random, so the
+//        sum of a block by less than 2^-56 of the sum of |phi . S|; binary64
+//        rounds the running sum 16 times a site.
+// A field of directions (|phi| about 1) has 2^55 and 2^53, a Gaussian one of
+// 2^24 sites 2^54 and 2^50.
+constexpr int kMeanBits = 52, kProductBits = 48;
 // From 2^20 sites the large bricks (4096 sites: fewer bonds leave them) and the
 // merge with several rows a warp; below, one site a thread and small bricks, so
 // that L = 16 still has 256 CTAs: 8 us against 20 with 8 x 4 x 4 x 4 bricks of
@@ -626,11 +684,11 @@ constexpr int64_t kLargeSites = 1 << 20;
 //
 // PROJECT: the same pass takes the projections of the next update, which read
 // the same field and are bound by the binary64 pipe while the sums are bound
-// by integer issue: 303 us together, 222 + 156 apart (L = 64).
+// by integer issue: 303 us together, 222 + 156 apart (L = 64, the 54-bit grid).
 template <bool PROJECT>
 __global__ void __launch_bounds__(kObserveThreads)
-    phi4_observe_fixed_kernel(const F4* phi, int L, int64_t n, const uint32_t* top, int steps, double* out, double* a,
-                              float* af, Dir d, uint32_t* next_top) {
+    phi4_observe_fixed_kernel(const F4* phi, int L, int64_t n, const uint32_t* top, int steps, double* part,
+                              uint32_t* done, double* out, double* a, float* af, Dir d, uint32_t* next_top) {
   sw::start_next();
   sw::after_previous();
   uint32_t big = 0u;
@@ -640,24 +698,29 @@ __global__ void __launch_bounds__(kObserveThreads)
     af[x] = __double2float_rn(v);
     big = max(max(max(big, abs_high(f.x)), abs_high(f.y)), max(abs_high(f.z), abs_high(f.w)));
   };
+  auto leave_top = [&] {
+    big = __reduce_max_sync(0xffffffffu, big);
+    if ((threadIdx.x & 31) == 0) atomicMax(next_top, big);
+  };
+  double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   const int et = (int)(*top >> 20);  // biased exponent of the largest component before the reflection
   if (et < 1023 - 400 || et > 1023 + 400) {
     // zero, subnormal, huge, infinite or NaN components: the binary64 sums
-    double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    const int64_t b = (int64_t)blockIdx.y * gridDim.x + blockIdx.x, x0 = b * blockDim.x + threadIdx.x,
+    const int64_t b = (int64_t)blockIdx.y * gridDim.x + blockIdx.x,
                   step = (int64_t)gridDim.x * gridDim.y * blockDim.x;
-    observe_binary64(phi, L, n, x0, step, v);
-    block_add5(v, out);
-    if (PROJECT) {
-      for (int64_t x = x0; x < n; x += step) project(phi[x], x);
-      big = __reduce_max_sync(0xffffffffu, big);
-      if ((threadIdx.x & 31) == 0) atomicMax(next_top, big);
+    for (int64_t x = b * blockDim.x + threadIdx.x; x < n; x += step) {
+      observe_site(phi, (uint32_t)L, (uint32_t)x, v);
+      if (PROJECT) project(phi[x], x);
     }
+    if (PROJECT) leave_top();
+    grid_sum5(v, part, done, out);
     return;
   }
   const int T = et - 1023 + 2;        // |phi| <= 2 max component < 2^T
-  const int shift0 = T + 1031;
+  const int shift0 = T + 1027;
   __shared__ longlong2 s_x[2][2][kObserveThreads];
+  __shared__ uint32_t s_chk[7];  // sums of |phi_c| and |phi . S| (2^-40), counts of components that lost bits
+  if (threadIdx.x < 7) s_chk[threadIdx.x] = 0u;  // (the loop's barriers follow)
   const uint32_t V = (uint32_t)L * L * L, s0 = blockIdx.x * kObserveThreads, s = s0 + threadIdx.x;
   const bool have = s < V;
   const uint32_t sc = have ? s : V - 1;
@@ -665,15 +728,16 @@ __global__ void __launch_bounds__(kObserveThreads)
   const uint32_t n0 = nb(sc, 0, k, L, 1), n1 = nb(sc, 1, k, L, L), n2 = sc + (k.c[2] + 1 == (uint32_t)L ? L * L - V : L * L);
   const bool in0 = n0 - s0 < kObserveThreads, in1 = n1 - s0 < kObserveThreads;
   const int z0 = blockIdx.y * steps, z1 = min(z0 + steps, L);
-  int64_t hh = 0, cr = 0, ll = 0, m[4] = {0, 0, 0, 0};
+  int64_t E = 0, m[4] = {0, 0, 0, 0};
+  uint32_t am[4] = {0u, 0u, 0u, 0u}, ae = 0u, own_lost, up_lost, nlost = 0u;  // high words of |.|; counts by byte
   const F4 first = phi[(size_t)z0 * V + sc];
   if (PROJECT && have) project(first, (size_t)z0 * V + sc);
-  Fix4 own = to_fixed(first, shift0);
+  Fix4 own = to_fixed(first, shift0, own_lost);
   for (int z = z0; z < z1; ++z) {
     const F4* slice = phi + (size_t)z * V;
     const F4 fu = phi[(size_t)(z + 1 == L ? 0 : z + 1) * V + sc];
     if (PROJECT && have && z + 1 < z1) project(fu, (size_t)(z + 1) * V + sc);
-    const Fix4 up = to_fixed(fu, shift0);
+    const Fix4 up = to_fixed(fu, shift0, up_lost);
     const F4 g2 = slice[n2];
     longlong2(&buf)[2][kObserveThreads] = s_x[z & 1];
     buf[0][threadIdx.x] = make_longlong2(own.v[0], own.v[1]);
@@ -695,31 +759,51 @@ __global__ void __launch_bounds__(kObserveThreads)
 #pragma unroll
       for (int c = 0; c < 4; ++c) S.v[c] += g.v[c];
     }
+    int64_t hh = 0, cr = 0, ll = 0;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const int xh = (int)(own.v[c] >> 27), Sh = (int)(S.v[c] >> 27);
-      const int xl = (int)own.v[c] & 0x7ffffff, Sl = (int)S.v[c] & 0x7ffffff;
+      const int xh = (int)(own.v[c] >> 30), Sh = (int)(S.v[c] >> 30);
+      const int xl = (int)own.v[c] & 0x3fffffff, Sl = (int)S.v[c] & 0x3fffffff;
       hh += (int64_t)xh * Sh;
       cr += (int64_t)xh * Sl + (int64_t)xl * Sh;
       ll += (int64_t)xl * Sl;
       m[c] += own.v[c];
+      am[c] += (uint32_t)abs((int)(own.v[c] >> 32));
     }
+    // phi . S = hh 2^60 + cr 2^30 + ll, to the nearest multiple of 2^60
+    const int64_t e = hh + ((cr + (ll >> 30) + (1 << 29)) >> 30);
+    E += e;
+    ae += (uint32_t)abs((int)(e >> 32));
+    nlost += own_lost;
     own = up;
+    own_lost = up_lost;
   }
-  double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  if (have) {
-    // E = hh 2^54 + cr 2^27 + ll, rounded to a multiple of 2^54 (2^-54 of a site's bound)
-    hh += (cr + ((ll + (1 << 26)) >> 27) + (1 << 26)) >> 27;
-    v[0] = (double)hh * scalbn(1.0, 2 * T - 54);
-    const double u = scalbn(1.0, T - 54);
+  {
+    const uint32_t w[7] = {am[0] >> 8, am[1] >> 8, am[2] >> 8, am[3] >> 8,
+                           ae >> 8,    nlost & 0x00ff00ffu, (nlost >> 8) & 0x00ff00ffu};
+#pragma unroll
+    for (int c = 0; c < 7; ++c) {
+      const uint32_t sum = __reduce_add_sync(0xffffffffu, have ? w[c] : 0u);
+      if ((threadIdx.x & 31) == 0) atomicAdd(&s_chk[c], sum);
+    }
+  }
+  __syncthreads();
+  const uint32_t sites = min((uint32_t)kObserveThreads, V - s0) * (uint32_t)(z1 - z0);
+  const bool fixed = s_chk[4] >= sites << (kProductBits - 40) &&
+                     s_chk[0] >= (s_chk[5] & 0xffffu) << (kMeanBits - 40) &&
+                     s_chk[1] >= (s_chk[6] & 0xffffu) << (kMeanBits - 40) &&
+                     s_chk[2] >= (s_chk[5] >> 16) << (kMeanBits - 40) &&
+                     s_chk[3] >= (s_chk[6] >> 16) << (kMeanBits - 40);  // the same in every thread
+  if (have && fixed) {
+    v[0] = (double)E * scalbn(1.0, 2 * T - 56);
+    const double u = scalbn(1.0, T - 58);
 #pragma unroll
     for (int c = 0; c < 4; ++c) v[1 + c] = (double)m[c] * u;
+  } else if (have) {
+    for (int z = z0; z < z1; ++z) observe_site(phi, (uint32_t)L, (uint32_t)z * V + s, v);
   }
-  block_add5(v, out);
-  if (PROJECT) {
-    big = __reduce_max_sync(0xffffffffu, big);
-    if ((threadIdx.x & 31) == 0) atomicMax(next_top, big);
-  }
+  if (PROJECT) leave_top();
+  grid_sum5(v, part, done, out);
 }
 
 int grid_of(int64_t n) {
@@ -752,6 +836,8 @@ struct sw_phi4 {
   uint8_t* bonds = nullptr;
   double* obs = nullptr;  // [cap][5]: E, M0..M3
   uint32_t* top = nullptr;  // [2], by update parity: high word of the field's largest |component| (projection -> E and M)
+  double* part = nullptr;   // large lattices: the blocks' E and M, [blocks][5]
+  uint32_t* done = nullptr;  // and the count of those that are in
   int* err = nullptr;
   sw::ReadBack read;
 };
@@ -768,7 +854,7 @@ namespace {
   } while (0)
 
 void free_phi4(sw_phi4* h) {
-  void* ptrs[] = {h->phi, h->a, h->af, h->par, h->bonds, h->obs, h->top, h->err};
+  void* ptrs[] = {h->phi, h->a, h->af, h->par, h->bonds, h->obs, h->top, h->part, h->done, h->err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -841,6 +927,11 @@ void launch_merge(sw_phi4* h) {
                    h->bonds, h->par, h->n, (uint32_t)h->t, h->ks, h->err);
 }
 
+dim3 observe_grid(int L) {
+  return dim3((unsigned)(((int64_t)L * L * L + kObserveThreads - 1) / kObserveThreads),
+              (unsigned)((L + kObserveSteps - 1) / kObserveSteps));
+}
+
 // The direction of update t and, on large lattices, its cleared range word.
 int begin_update(sw_phi4* h, int64_t t, Dir& d) {
   if (direction(h->seed, (uint32_t)t, d) != 0) return ffail(SW_EDEVICE, "no direction found");
@@ -911,6 +1002,12 @@ int sw_phi4_create(int32_t L, double kappa, uint64_t seed, int32_t init, void* s
   if (e == cudaSuccess) e = cudaMalloc(&h->par, n * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->bonds, n);
   if (e == cudaSuccess) e = cudaMalloc(&h->top, 2 * sizeof(uint32_t));
+  if (e == cudaSuccess && h->n >= kLargeSites) {
+    const dim3 g = observe_grid(L);
+    e = cudaMalloc(&h->part, (size_t)g.x * g.y * 5 * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&h->done, sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->done, 0, sizeof(uint32_t), h->stream);
+  }
   if (e == cudaSuccess) e = cudaMalloc(&h->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int), h->stream);
   if (e == cudaSuccess) {
@@ -941,8 +1038,7 @@ int sw_phi4_sweep(sw_phi4* h, int32_t n) {
   if (n == 0) return SW_OK;
   const int g = grid_of(h->n), L = h->L;
   const bool large = h->n >= kLargeSites;
-  const dim3 og((unsigned)(((int64_t)L * L * L + kObserveThreads - 1) / kObserveThreads),
-                (unsigned)((L + kObserveSteps - 1) / kObserveSteps));
+  const dim3 og = observe_grid(L);
   Dir d, next{};
   rc = begin_update(h, h->t, d);
   if (rc != SW_OK) return rc;
@@ -963,10 +1059,10 @@ int sw_phi4_sweep(sw_phi4* h, int32_t n) {
     }
     if (large && more)
       sw::launch_after(phi4_observe_fixed_kernel<true>, og, kObserveThreads, 0, h->stream, h->phi, L, h->n, top,
-                       kObserveSteps, o, h->a, h->af, next, h->top + ((h->t + 1) & 1));
+                       kObserveSteps, h->part, h->done, o, h->a, h->af, next, h->top + ((h->t + 1) & 1));
     else if (large)
       sw::launch_after(phi4_observe_fixed_kernel<false>, og, kObserveThreads, 0, h->stream, h->phi, L, h->n, top,
-                       kObserveSteps, o, nullptr, nullptr, d, nullptr);
+                       kObserveSteps, h->part, h->done, o, nullptr, nullptr, d, nullptr);
     else
       sw::launch_after(phi4_observe_kernel, g, 256, 0, h->stream, h->phi, L, h->n, o);
     F_CUDA(cudaGetLastError(), "phi4 reflect launch");
