@@ -115,9 +115,10 @@ __device__ __forceinline__ uint32_t nb(uint32_t x, int mu, const Coords& k, uint
 // and w < (1 - e^{-z}) 2^32 with z = k4 q, all in binary64 with exp_neg.
 // GB300 runs binary64 at a small fraction of its binary32 rate, so a
 // binary32 estimate decides first, from the projections rounded to binary32
-// (af, each within 2^-24 relative): with both |af| >= 2^-60 the estimate of z
-// (three roundings of 2^-24 and two products) is within 5 * 2^-24 relative and
-// has the sign of q, so for 0 < z <= 40 e^{-z} from expf (2 ulp) is within
+// (af, each within 2^-24 relative): with both |af| >= 2^-60 and k4 >= 2^-66
+// (k4 af is then a normal number; smaller couplings come as NaN) the estimate
+// of z (three roundings of 2^-24 and two products) is within 5 * 2^-24 relative,
+// or below 2^-126 with z, and has the sign of q, so for 0 < z <= 40 e^{-z} from expf (2 ulp) is within
 // 40 * 5 * 2^-24 + 2^-22 of the binary64 value and (1 - e) 2^32 within 2^16 of
 // the binary64 threshold; beyond 40 both thresholds are 2^32 to binary32
 // precision, and for z < 0 the estimate is not positive. A word more than 2^18
@@ -281,7 +282,9 @@ __global__ void __launch_bounds__(NT)
   float* const s_af = reinterpret_cast<float*>(s_buf);  // [V] projections, then the warps' lists
   __shared__ int s_par[V];
   __shared__ uint8_t s_b[V];  // bits 0-3: bonds inside the brick, 4-7: bonds that leave it
-  const float k4f = __double2float_rn(k4);
+  // (k4 f) f stays in binary32's normal range, or vanishes, for |f| >= 2^-60
+  // unless k4 is below 2^-66: with NaN every edge takes the binary64 test
+  const float k4f = k4 == 0.0 || k4 >= 0x1p-66 ? __double2float_rn(k4) : __int_as_float(0x7fffffff);
   const uint32_t uL = (uint32_t)L, L2 = uL * uL, L3 = L2 * uL;
   uint32_t q = blockIdx.x;
   const uint32_t g0 = (uL + B0 - 1) / B0, g1 = (uL + B1 - 1) / B1, g2 = (uL + B2 - 1) / B2;
