@@ -1617,11 +1617,15 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
   if (HIST) {
     // sizes are complete after this barrier: bin the inner clusters (the
     // tile roots phase 1 marked, less the border roots), send border pieces
-    // to their global root. Counts, sums of squares (at most 8192^2 a tile)
-    // and bins 0-7 (8-bit fields: at most 64 roots a thread) add up in
-    // registers and once per warp into the shared histogram.
+    // to their global root. Counts, sums of squares (at most 16384^2 a tile)
+    // and bins 0-7 add up in registers and once per warp into the shared
+    // histogram. A thread can meet 32 H roots, all in one bin (beta = 0: every
+    // site its own cluster), so the bins take 8-bit fields up to four rows a
+    // strip and 16-bit fields above.
     __syncthreads();
-    uint32_t cnt = 0u, sq = 0u, bins03 = 0u, bins47 = 0u;
+    constexpr int BF = 32 * H <= 255 ? 8 : 16, PW = 32 / BF;  // bits a bin, bins a word
+    static_assert(32 * H < (1 << BF) && TH * TW <= 16384, "bins and sums of squares hold");
+    uint32_t cnt = 0u, sq = 0u, bins[8 / PW] = {};
 #pragma unroll
     for (int r = 0; r < H; ++r) {
       if (r >= nv || !wmask) continue;
@@ -1637,9 +1641,13 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
           const int bin = log2_floor(sz);
           cnt += 1u;
           sq += sz * sz;
-          if (bin < 4) bins03 += 1u << (8 * bin);
-          else if (bin < 8) bins47 += 1u << (8 * (bin - 4));
-          else atomicAdd(&s_hist[2 + bin], 1ull);
+          if (bin < 8) {
+#pragma unroll
+            for (int q = 0; q < 8 / PW; ++q)
+              if (bin / PW == q) bins[q] += 1u << (BF * (bin % PW));
+          } else {
+            atomicAdd(&s_hist[2 + bin], 1ull);
+          }
         }
       }
     }
@@ -1648,10 +1656,8 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
     sq = __reduce_add_sync(0xffffffffu, sq);
     uint32_t bsum[8];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      bsum[q] = __reduce_add_sync(0xffffffffu, (bins03 >> (8 * q)) & 0xffu);
-      bsum[4 + q] = __reduce_add_sync(0xffffffffu, (bins47 >> (8 * q)) & 0xffu);
-    }
+    for (int q = 0; q < 8; ++q)
+      bsum[q] = __reduce_add_sync(0xffffffffu, (bins[q / PW] >> (BF * (q % PW))) & ((1u << BF) - 1u));
     if (lane == 0) {
       if (cnt) atomicAdd(&s_hist[0], (unsigned long long)cnt);
       if (sq) atomicAdd(&s_hist[1], (unsigned long long)sq);
