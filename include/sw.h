@@ -70,6 +70,10 @@
  *    to the host (sw_observables, sw_histograms, host-buffer forms of
  *    sw_labels/sw_spins/sw_bonds) synchronise that stream and check the
  *    device error flag (SW_EDEVICE / SW_ETIMEOUT).
+ *  - Several host threads may read the trace of one handle at the same time
+ *    (sw_observables, sw_histograms, and the observables of batches, Potts
+ *    lattices and phi^4 fields); every other use of a handle from several
+ *    threads is the caller's to serialise. Different handles are independent.
  *  - There is no CPU fallback: without a usable GPU, sw_create returns
  *    SW_ECUDA.
  */

@@ -111,6 +111,7 @@ __global__ void read_back_kernel(const int* err, const unsigned long long* src, 
 }  // namespace
 
 cudaError_t ReadBack::operator()(cudaStream_t st, const int* err, const void* src, size_t words, int* flag, void* out) {
+  std::lock_guard<std::mutex> turn(mutex_);
   if (!page_) {
     const cudaError_t e = cudaHostAlloc(&page_, kPageWords * sizeof *page_, cudaHostAllocDefault);
     if (e != cudaSuccess) return e;

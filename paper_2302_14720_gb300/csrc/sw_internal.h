@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "sw_philox.cuh"
 
 namespace sw {
@@ -161,7 +163,8 @@ struct BatchArgs {
 // on the stream, and one synchronisation ends the read: a stream wait and two
 // blocking copies took 16 us a read where this takes 7 (a batch of 256
 // replicas reads 256 traces). Longer stretches than the page are copied after
-// the flag.
+// the flag. Reads of one handle from several host threads take turns at its
+// page.
 class ReadBack {
  public:
   ReadBack() = default;
@@ -176,6 +179,7 @@ class ReadBack {
 
  private:
   static constexpr size_t kPageWords = 4096;
+  std::mutex mutex_;
   unsigned long long* page_ = nullptr;
 };
 
