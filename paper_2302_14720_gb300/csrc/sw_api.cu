@@ -112,6 +112,15 @@ __global__ void read_back_kernel(const int* err, const unsigned long long* src, 
 
 cudaError_t ReadBack::operator()(cudaStream_t st, const int* err, const void* src, size_t words, int* flag, void* out) {
   std::lock_guard<std::mutex> turn(mutex_);
+  int current = device_;
+  cudaError_t e = cudaGetDevice(&current);
+  if (e == cudaSuccess && current != device_ && device_ >= 0) e = cudaSetDevice(device_);
+  if (e == cudaSuccess) e = read(st, err, src, words, flag, out);
+  if (current != device_ && device_ >= 0) cudaSetDevice(current);
+  return e;
+}
+
+cudaError_t ReadBack::read(cudaStream_t st, const int* err, const void* src, size_t words, int* flag, void* out) {
   if (!page_) {
     const cudaError_t e = cudaHostAlloc(&page_, kPageWords * sizeof *page_, cudaHostAllocDefault);
     if (e != cudaSuccess) return e;

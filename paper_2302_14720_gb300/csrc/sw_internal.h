@@ -164,10 +164,13 @@ struct BatchArgs {
 // blocking copies took 16 us a read where this takes 7 (a batch of 256
 // replicas reads 256 traces). Longer stretches than the page are copied after
 // the flag. Reads of one handle from several host threads take turns at its
-// page.
+// page, and any device may be current: the kernel is launched on the one that
+// was when the handle was created.
 class ReadBack {
  public:
-  ReadBack() = default;
+  ReadBack() {
+    if (cudaGetDevice(&device_) != cudaSuccess) device_ = -1;
+  }
   ReadBack(const ReadBack&) = delete;
   ReadBack& operator=(const ReadBack&) = delete;
   ~ReadBack() {
@@ -179,7 +182,9 @@ class ReadBack {
 
  private:
   static constexpr size_t kPageWords = 4096;
+  cudaError_t read(cudaStream_t st, const int* err, const void* src, size_t words, int* flag, void* out);
   std::mutex mutex_;
+  int device_ = -1;
   unsigned long long* page_ = nullptr;
 };
 
