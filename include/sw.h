@@ -252,7 +252,9 @@ typedef struct sw_batch sw_batch;
 
 /* Create a batch with n >= 0 replicas (side L[i], beta[i], seed[i], init[i]
  * or SW_INIT_HOT when init is NULL). shape: a compiled tile shape index or
- * -1 for the default. stream: as for sw_create. The batch owns all device
+ * -1 for the default (sw_tune_shape), which follows the replicas: a batch on
+ * 128x32 tiles that outgrows them is laid out anew by sw_batch_add (which then
+ * synchronises the stream). stream: as for sw_create. The batch owns all device
  * memory of its replicas. Errors: SW_EINVAL, SW_ENOMEM, SW_ECUDA. */
 int sw_batch_create(int32_t n, const int32_t* L, const double* beta, const uint64_t* seed,
                     const int32_t* init, int32_t shape, void* stream, sw_batch** out);

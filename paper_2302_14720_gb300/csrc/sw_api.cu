@@ -64,9 +64,8 @@ int bucket_of(int L) {
   return b < kBuckets ? b : kBuckets - 1;
 }
 
-// lattice: the shape of a lone lattice (sw_create); else of a batch whose
-// largest side is L.
-int shape_for(int L, bool lattice, int64_t batch_tiles = 0) {
+// The shape of SW_TILE_SHAPE or of the tuned entry of L's size bucket; -1: none.
+int preferred_shape(int L) {
   if (const char* env = getenv("SW_TILE_SHAPE")) {
     const int v = atoi(env);
     if (v >= 0 && v < sw::kNumShapes) return v;
@@ -74,27 +73,32 @@ int shape_for(int L, bool lattice, int64_t batch_tiles = 0) {
   std::call_once(g_tuned_once, [] {
     for (auto& x : g_tuned) x.store(-1);
   });
-  const int t = g_tuned[bucket_of(L)].load();
-  if (t >= 0) return t;
-  // A lone lattice of side <= 1024 has at most 128 tiles of 128 x 64, less
-  // than one wave of 152 SMs; with 128 x 32 tiles twice as many CTAs share
-  // each phase's latency, and in phase 3 a thread has one row word (one-row
-  // strips) instead of two to walk. With these strips phases 1 and 3 take the
-  // same block, so that chains run them in one launch: L = 256 44.5 -> 36.7
-  // us a sweep, 1024 49.9 -> 40.3, with statistics 78 -> 64.
-  if (lattice) return L <= 1024 ? 7 : 6;
-  // A batch by the same rule as long as its replicas have at most four 128 x
-  // 64 tiles an SM (8 replicas up to L = 64 55 -> 38 us a sweep, 128 replicas
-  // up to 256, 470 tiles, 114 -> 106), 128 x 64 tiles above (256 replicas up
-  // to 1024, 9100 tiles, 573 against 643).
-  if (batch_tiles > 0 && batch_tiles <= 4 * 152) return 7;
-  return L <= 64 ? 2 : 6;
+  return g_tuned[bucket_of(L)].load();
+}
+
+// A lone lattice of side <= 1024 has at most 128 tiles of 128 x 64, less
+// than one wave of 152 SMs; with 128 x 32 tiles twice as many CTAs share
+// each phase's latency, and in phase 3 a thread has one row word (one-row
+// strips) instead of two to walk. With these strips phases 1 and 3 take the
+// same block, so that chains run them in one launch: L = 256 44.5 -> 36.7
+// us a sweep, 1024 49.9 -> 40.3, with statistics 78 -> 64.
+int lattice_shape(int L) {
+  const int p = preferred_shape(L);
+  return p >= 0 ? p : L <= 1024 ? 7 : 6;
 }
 
 }  // namespace
 
 namespace sw {
-int default_shape(int L, int64_t tiles) { return shape_for(L, false, tiles); }
+// Batches by the same rule as lone lattices, as long as their replicas have
+// at most four 128 x 64 tiles an SM (8 replicas up to L = 64 55 -> 38 us a
+// sweep, 128 replicas up to 256, 470 tiles, 114 -> 106), 128 x 64 tiles above
+// (256 replicas up to 1024, 9100 tiles, 573 against 643).
+int builtin_batch_shape(int L, int64_t tiles) {
+  if (tiles > 0 && tiles <= 4 * 152) return kSmallBatchShape;
+  return L <= 64 ? 2 : 6;
+}
+int preferred_batch_shape(int L) { return preferred_shape(L); }
 }  // namespace sw
 
 namespace sw {
@@ -379,7 +383,7 @@ int sw_create(int32_t L, double beta, uint64_t seed, int32_t init, void* stream,
   h->beta = beta;
   h->seed = seed;
   h->thr = threshold_of(beta);
-  h->shape = shape_for(L, true);
+  h->shape = lattice_shape(L);
   h->tiles_only = getenv("SW_TILE_SHAPE") != nullptr;
   h->ks = sw::make_key_schedule(seed);
   cudaGetDevice(&h->device);
@@ -665,7 +669,7 @@ int sw_shape_info(int32_t shape, int32_t* tile_w, int32_t* tile_h, int32_t* stri
 int sw_tune_shape(int32_t log2_bucket, int32_t shape) {
   if (log2_bucket < 0 || log2_bucket >= kBuckets) return fail(SW_EINVAL, "bucket must be in [0, %d)", kBuckets);
   if (shape < -1 || shape >= sw::kNumShapes) return fail(SW_EINVAL, "unknown tile shape %d", shape);
-  shape_for(2, true);  // initialise the table
+  preferred_shape(2);  // initialise the table
   g_tuned[log2_bucket].store(shape);
   return SW_OK;
 }

@@ -39,6 +39,7 @@ struct Replica {
   bool small = false;  // on the one-CTA path (L <= the batch's small_max_L)
   int8_t* spins = nullptr;
   sw::TileBuffers tb{};
+  sw::TileBuffers next{};  // the buffers of a new shape while the batch is laid out anew
   int64_t* em = nullptr;
 };
 
@@ -49,10 +50,37 @@ uint32_t thr_of(double beta) {
   return (uint32_t)scaled;
 }
 
-void free_replica(Replica& r) {
-  void* ptrs[] = {r.spins, r.tb.tbits, r.tb.roots, r.tb.bmask, r.tb.rbits, r.tb.nodes, r.tb.bslot, r.tb.bbits, r.tb.nslots, r.em};
+void free_tiles(sw::TileBuffers& tb) {
+  void* ptrs[] = {tb.tbits, tb.roots, tb.bmask, tb.rbits, tb.nodes, tb.bslot, tb.bbits, tb.nslots};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  tb = sw::TileBuffers{};
+}
+
+int tiles_of(const sw::TileShape& ts, int L) {
+  return ((L + ts.tw() - 1) / ts.tw()) * ((L + ts.th - 1) / ts.th);
+}
+
+// The tile buffers of a replica of side L; on an error some are allocated.
+cudaError_t alloc_tiles(sw::TileBuffers& tb, const sw::TileShape& ts, int L, int* err) {
+  const size_t nt = (size_t)tiles_of(ts, L);
+  cudaError_t e = cudaMalloc(&tb.tbits, nt * 3 * ts.row_words() * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&tb.roots, nt * ts.sites() * sizeof(uint16_t));
+  if (e == cudaSuccess) e = cudaMalloc(&tb.bmask, nt * ts.row_words() * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&tb.rbits, nt * ts.row_words() * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&tb.nodes, nt * ts.max_slots() * sizeof(uint64_t));
+  if (e == cudaSuccess) e = cudaMalloc(&tb.bslot, nt * ts.boundary_sites() * sizeof(uint16_t));
+  if (e == cudaSuccess) e = cudaMalloc(&tb.bbits, nt * ts.bbits_words() * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&tb.nslots, nt * sizeof(int32_t));
+  tb.err = err;
+  return e;
+}
+
+void free_replica(Replica& r) {
+  free_tiles(r.tb);
+  free_tiles(r.next);
+  if (r.spins) cudaFree(r.spins);
+  if (r.em) cudaFree(r.em);
   r = Replica{};
 }
 
@@ -60,7 +88,7 @@ void free_replica(Replica& r) {
 
 struct sw_batch {
   int shape = 0;
-  bool own_shape = false;  // the library chose the shape
+  bool own_shape = false;  // the built-in choice, which follows the replicas
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int* d_err = nullptr;
@@ -252,6 +280,45 @@ int64_t replica_bytes(const sw::TileShape& ts, int L, int64_t cap) {
          cap * 16;
 }
 
+// The shape the built-in choice gives the batch with one more replica of side
+// L (0: as it is): a batch on kSmallBatchShape leaves it when it has outgrown it.
+int shape_with(const sw_batch* b, int L) {
+  if (!b->own_shape || b->shape != sw::kSmallBatchShape) return b->shape;
+  const sw::TileShape ts = sw::shape_of(6);
+  int lmax = L > 2 ? L : 2;
+  int64_t tiles = L > 0 ? tiles_of(ts, L) : 0;
+  for (const Replica& r : b->reps) {
+    if (!r.active) continue;
+    lmax = r.L > lmax ? r.L : lmax;
+    tiles += tiles_of(ts, r.L);
+  }
+  return sw::builtin_batch_shape(lmax, tiles);
+}
+
+// Lays the batch out on tiles of another shape: new tile buffers for every
+// replica (they hold nothing between sweeps). Nothing changes on an error.
+int set_shape(sw_batch* b, int shape) {
+  if (shape == b->shape) return SW_OK;
+  const sw::TileShape ts = sw::shape_of(shape);
+  B_CUDA(cudaStreamSynchronize(b->stream), "stream synchronize");
+  cudaError_t e = cudaSuccess;
+  for (Replica& r : b->reps)
+    if (r.active && e == cudaSuccess) e = alloc_tiles(r.next, ts, r.L, b->d_err);
+  for (Replica& r : b->reps) {
+    if (!r.active) continue;
+    if (e == cudaSuccess) {
+      std::swap(r.tb, r.next);
+      r.ntiles = tiles_of(ts, r.L);
+    }
+    free_tiles(r.next);
+  }
+  if (e != cudaSuccess) return cuda_bfail(e, "tile buffers of a new shape");
+  drop_graph(b);
+  b->shape = shape;
+  b->dirty = true;
+  return SW_OK;
+}
+
 int check_slot(sw_batch* b, int32_t slot) {
   if (!b) return bfail(SW_EINVAL, "batch is NULL");
   if (slot < 0 || slot >= (int32_t)b->reps.size() || !b->reps[slot].active)
@@ -294,8 +361,9 @@ int sw_batch_create(int32_t n, const int32_t* L, const double* beta, const uint6
       lmax = L[i] > lmax ? L[i] : lmax;
       if (L[i] >= 2) tiles += ((int64_t)L[i] + 127) / 128 * (((int64_t)L[i] + 63) / 64);
     }
-    shape = sw::default_shape(lmax, tiles);
-    b->own_shape = true;
+    shape = sw::preferred_batch_shape(lmax);
+    b->own_shape = shape < 0;
+    if (shape < 0) shape = sw::builtin_batch_shape(lmax, tiles);
   }
   b->shape = shape;
   cudaError_t e = cudaSuccess;
@@ -331,30 +399,23 @@ int sw_batch_add(sw_batch* b, int32_t L, double beta, uint64_t seed, int32_t ini
   if (L < 2 || (int64_t)L * L >= ((int64_t)1 << 31)) return bfail(SW_EINVAL, "L outside 2 <= L, L*L < 2^31");
   if (!(beta >= 0.0) || isinf(beta)) return bfail(SW_EINVAL, "beta must be finite and >= 0");
   if (init != SW_INIT_HOT && init != SW_INIT_COLD) return bfail(SW_EINVAL, "init must be SW_INIT_HOT or SW_INIT_COLD");
+  int rc = set_shape(b, shape_with(b, L));
+  if (rc != SW_OK) return rc;
   const sw::TileShape ts = sw::shape_of(b->shape);
   Replica r;
   r.L = L;
   r.beta = beta;
   r.seed = seed;
   r.thr = thr_of(beta);
-  r.ntiles = ((L + ts.tw() - 1) / ts.tw()) * ((L + ts.th - 1) / ts.th);
-  const size_t nt = (size_t)r.ntiles, N = (size_t)L * L;
-  cudaError_t e = cudaMalloc(&r.spins, N);
-  if (e == cudaSuccess) e = cudaMalloc(&r.tb.tbits, nt * 3 * ts.row_words() * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&r.tb.roots, nt * ts.sites() * sizeof(uint16_t));
-  if (e == cudaSuccess) e = cudaMalloc(&r.tb.bmask, nt * ts.row_words() * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&r.tb.rbits, nt * ts.row_words() * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&r.tb.nodes, nt * ts.max_slots() * sizeof(uint64_t));
-  if (e == cudaSuccess) e = cudaMalloc(&r.tb.bslot, nt * ts.boundary_sites() * sizeof(uint16_t));
-  if (e == cudaSuccess) e = cudaMalloc(&r.tb.bbits, nt * ts.bbits_words() * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&r.tb.nslots, nt * sizeof(int32_t));
+  r.ntiles = tiles_of(ts, L);
+  cudaError_t e = cudaMalloc(&r.spins, (size_t)L * L);
+  if (e == cudaSuccess) e = alloc_tiles(r.tb, ts, L, b->d_err);
   if (e == cudaSuccess) e = sw::launch_init(r.spins, L, seed, init == SW_INIT_COLD, b->stream);
   if (e != cudaSuccess) {
     free_replica(r);
     return cuda_bfail(e, "sw_batch_add");
   }
-  r.tb.err = b->d_err;
-  const int rc = grow_trace(r, 1024, b->stream);
+  rc = grow_trace(r, 1024, b->stream);
   if (rc != SW_OK) {
     free_replica(r);
     return rc;
@@ -565,7 +626,13 @@ int sw_batch_footprint(sw_batch* b, int32_t L, int64_t sweeps, int64_t* bytes) {
   if (!b || !bytes) return bfail(SW_EINVAL, "NULL argument");
   if (L < 2 || (int64_t)L * L >= ((int64_t)1 << 31)) return bfail(SW_EINVAL, "L outside 2 <= L, L*L < 2^31");
   if (sweeps < 0) return bfail(SW_EINVAL, "sweeps must be >= 0");
-  *bytes = replica_bytes(sw::shape_of(b->shape), L, trace_cap_for(sweeps));
+  const int shape = shape_with(b, L);
+  const sw::TileShape ts = sw::shape_of(shape);
+  int64_t more = 0;  // what the present replicas take in addition if this one changes the shape
+  if (shape != b->shape)
+    for (const Replica& r : b->reps)
+      if (r.active) more += replica_bytes(ts, r.L, r.cap) - replica_bytes(sw::shape_of(b->shape), r.L, r.cap);
+  *bytes = replica_bytes(ts, L, trace_cap_for(sweeps)) + (more > 0 ? more : 0);
   return SW_OK;
 }
 

@@ -191,11 +191,14 @@ class ReadBack {
 // Set the thread's last error message (sw_last_error) and return code.
 int record_error(int code, const char* msg);
 
-// Tile shape for a lattice of side L: SW_TILE_SHAPE override, else the
-// tuned entry of L's size bucket, else the built-in default.
-// For a batch, L is the largest side and `tiles` the 128 x 64 tiles of its
-// replicas (0: none yet).
-int default_shape(int L, int64_t tiles);
+// Tile shapes of batches created without one: the preference for its largest
+// side L (SW_TILE_SHAPE, else the tuned entry of L's size bucket; -1: none),
+// else the built-in choice, by L and the 128 x 64 tiles of all replicas (0:
+// none yet). kSmallBatchShape is taken for few tiles only: a batch that grows
+// past them is laid out anew.
+constexpr int kSmallBatchShape = 7;
+int preferred_batch_shape(int L);
+int builtin_batch_shape(int L, int64_t tiles);
 
 // Launchers (sw_kernels.cu). Each returns cudaGetLastError() of its launches.
 cudaError_t launch_init(int8_t* spins, int L, uint64_t seed, int cold, cudaStream_t st);
