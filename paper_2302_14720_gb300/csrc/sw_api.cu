@@ -59,9 +59,9 @@ std::atomic<int> g_tuned[kBuckets];
 std::once_flag g_tuned_once;
 
 int bucket_of(int L) {
-  int b = 0;
-  while ((1 << b) < L) ++b;
-  return b < kBuckets ? b : kBuckets - 1;
+  int b = 0;  // (a side past the limit, not refused yet, goes to the last bucket)
+  while (b < kBuckets - 1 && (1 << b) < L) ++b;
+  return b;
 }
 
 // The shape of SW_TILE_SHAPE or of the tuned entry of L's size bucket; -1: none.
