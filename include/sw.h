@@ -291,9 +291,11 @@ int sw_batch_set_rule(sw_batch* b, int32_t slot, int32_t rule);
  *     SW_ETIMEOUT from the next synchronising call), captured as a CUDA
  *     graph with the barrier's reset (or launched directly where the
  *     cooperative launch cannot be captured).
- * The fused schedule needs a tile shape whose phases 1 and 3 run the same
- * block (64-row tiles of 2-row strips, 128-row tiles of 4-row strips):
- * SW_EINVAL otherwise. Synchronises the stream when the schedule changes. */
+ * The fused schedule needs 64-row tiles of 2-row strips or 128-row tiles of
+ * 4-row strips: SW_EINVAL otherwise. A batch on the built-in default's 128x32
+ * tiles moves to the tiles the default has for large batches (128x64; 64x64,
+ * without this schedule, if all sides are at most 64). Synchronises the stream
+ * when the schedule changes. */
 #define SW_SCHEDULE_PHASES 0
 #define SW_SCHEDULE_FUSED 1
 int sw_batch_set_schedule(sw_batch* b, int32_t schedule);

@@ -11,6 +11,7 @@
 #include <stdint.h>
 #include <stdlib.h>
 
+#include <algorithm>
 #include <climits>
 
 #include <cstdio>
@@ -280,19 +281,22 @@ int64_t replica_bytes(const sw::TileShape& ts, int L, int64_t cap) {
          cap * 16;
 }
 
+int largest_side(const sw_batch* b) {
+  int L = 2;
+  for (const Replica& r : b->reps)
+    if (r.active && r.L > L) L = r.L;
+  return L;
+}
+
 // The shape the built-in choice gives the batch with one more replica of side
-// L (0: as it is): a batch on kSmallBatchShape leaves it when it has outgrown it.
+// L: a batch on kSmallBatchShape leaves it when it has outgrown it.
 int shape_with(const sw_batch* b, int L) {
   if (!b->own_shape || b->shape != sw::kSmallBatchShape) return b->shape;
   const sw::TileShape ts = sw::shape_of(6);
-  int lmax = L > 2 ? L : 2;
-  int64_t tiles = L > 0 ? tiles_of(ts, L) : 0;
-  for (const Replica& r : b->reps) {
-    if (!r.active) continue;
-    lmax = r.L > lmax ? r.L : lmax;
-    tiles += tiles_of(ts, r.L);
-  }
-  return sw::builtin_batch_shape(lmax, tiles);
+  int64_t tiles = tiles_of(ts, L);
+  for (const Replica& r : b->reps)
+    if (r.active) tiles += tiles_of(ts, r.L);
+  return sw::builtin_batch_shape(std::max(L, largest_side(b)), tiles);
 }
 
 // Lays the batch out on tiles of another shape: new tile buffers for every
@@ -539,8 +543,15 @@ int sw_batch_set_schedule(sw_batch* b, int32_t schedule) {
   if (!b) return bfail(SW_EINVAL, "batch is NULL");
   if (schedule != SW_SCHEDULE_PHASES && schedule != SW_SCHEDULE_FUSED)
     return bfail(SW_EINVAL, "schedule must be SW_SCHEDULE_PHASES or SW_SCHEDULE_FUSED");
-  if (schedule == SW_SCHEDULE_FUSED && !sw::batch_fused_supported(b->shape, b->own_shape))
-    return bfail(SW_EINVAL, "the fused schedule needs a tile shape whose phases 1 and 3 take the same block");
+  if (schedule == SW_SCHEDULE_FUSED) {
+    // the built-in choice takes the tiles of a large batch for this schedule
+    int shape = b->shape;
+    if (b->own_shape && shape == sw::kSmallBatchShape) shape = sw::builtin_batch_shape(largest_side(b), 0);
+    if (!sw::batch_fused_supported(shape))
+      return bfail(SW_EINVAL, "the fused schedule needs 64-row tiles of 2-row strips or 128-row tiles of 4-row strips");
+    const int rc = set_shape(b, shape);
+    if (rc != SW_OK) return rc;
+  }
   if (schedule != b->schedule) {
     B_CUDA(cudaStreamSynchronize(b->stream), "stream synchronize");
     drop_graph(b);

@@ -218,9 +218,9 @@ cudaError_t launch_batch_advance(const BatchArgs& b, cudaStream_t st);
 // Batch, fused schedule: one cooperative launch runs nsweeps whole sweeps of
 // every replica with tiles (all four phases, grid barriers between them) and
 // advances the replicas' counters itself. Only shapes whose phases 1 and 3
-// take the same block (TH == 32 H) have it, and 128 x 32 only where the
-// library chose that shape.
-bool batch_fused_supported(int shape, bool own_shape);
+// take the same block (TH == 32 H) and whose tiles have 64 rows or more have
+// it: batch_fused_supported.
+bool batch_fused_supported(int shape);
 // Phase 3 of sweep t (a3) and phase 1 of sweep t + 1 (a1) in one launch, the
 // new spins handed over in shared memory (flip or assignment rule, no
 // statistics). Shapes whose phases 1 and 3 take the same block.

@@ -2303,16 +2303,13 @@ bool phase31_supported(int shape) {
   return shape >= 0 && shape < kNumShapes && shape_of(shape).th == 32 * shape_of(shape).h;
 }
 
-bool batch_fused_supported(int shape, bool own_shape) {
-  return phase31_supported(shape) && (own_shape || shape_of(shape).th >= 64);
-}
+bool batch_fused_supported(int shape) { return phase31_supported(shape) && shape_of(shape).th >= 64; }
 
 cudaError_t launch_batch_fused(int shape, const BatchArgs& b, int ntiles, int nsweeps, cudaStream_t st) {
   if (ntiles <= 0 || nsweeps <= 0) return cudaSuccess;
   switch (shape) {
     case 4: return launch_fused_shape<shape_of(4).wpr, shape_of(4).th, shape_of(4).h>(b, ntiles, nsweeps, st);
     case 6: return launch_fused_shape<shape_of(6).wpr, shape_of(6).th, shape_of(6).h>(b, ntiles, nsweeps, st);
-    case 7: return launch_fused_shape<shape_of(7).wpr, shape_of(7).th, shape_of(7).h>(b, ntiles, nsweeps, st);
   }
   return cudaErrorInvalidValue;
 }
