@@ -134,9 +134,9 @@ int sw_destroy(sw_lattice* h);
  * sweep E and M (C10), and the C11 statistics if enabled, are appended to
  * the device-side trace. Errors: SW_EINVAL (n < 0), SW_ENOMEM (trace
  * growth), SW_ECUDA. Device-side failures are reported by the next call that
- * synchronises. A lattice with L <= 160 (144 for n = 1) and statistics off
- * runs all n sweeps in one CTA-sized launch (the whole lattice in shared memory)
- * unless the environment variable SW_TILE_SHAPE was set at sw_create, which
+ * synchronises. A small lattice (L up to 96 .. 156, by n and the rule) with
+ * statistics off runs all n sweeps in one CTA-sized launch (the whole lattice
+ * in shared memory) unless the environment variable SW_TILE_SHAPE was set at sw_create, which
  * keeps it on the tiled path; the results are the same. Between the sweeps
  * of one call the bond draws of the next sweep (C5: they depend on the
  * seed, the counter and the site, not on the spins) are taken during the
@@ -500,8 +500,8 @@ int sw_shape_info(int32_t shape, int32_t* tile_w, int32_t* tile_h, int32_t* stri
  * shape. */
 int sw_tune_shape(int32_t log2_bucket, int32_t shape);
 
-/* The tile shape index a lattice was created with (its tiled path; sides up
- * to 160 run whole sweeps in one CTA unless SW_TILE_SHAPE is set). */
+/* The tile shape index a lattice was created with (its tiled path; small sides
+ * run whole sweeps in one CTA unless SW_TILE_SHAPE is set, see sw_sweep). */
 int sw_lattice_shape(sw_lattice* h, int32_t* shape);
 
 /* Message of the last failed call on this thread ("" if none). */

@@ -452,7 +452,7 @@ int sw_sweep(sw_lattice* h, int32_t n) {
   if (rc != SW_OK) return rc;
   const sw::TileShape ts = sw::shape_of(h->shape);
   (void)ts;
-  if (sw::small_sweep(h->L, n) && !h->hist_on && !h->tiles_only) {
+  if (h->L <= sw::small_sweep_max_L(n, h->rule == SW_RULE_ASSIGN) && !h->hist_on && !h->tiles_only) {
     // the whole lattice fits one CTA: all n sweeps in one launch
     sw::SmallArgs s{};
     s.L = h->L;

@@ -228,19 +228,29 @@ bool phase31_supported(int shape);
 cudaError_t launch_phase31(int shape, const SweepArgs& a3, const SweepArgs& a1, cudaStream_t st);
 cudaError_t launch_batch_fused(int shape, const BatchArgs& b, int ntiles, int nsweeps, cudaStream_t st);
 
-// Whole sweeps of one small lattice in one CTA (sw_small.cu). 181^2 < 2^15,
-// so 16-bit parents index every site.
+// Whole sweeps of one small lattice in one CTA (sw_small.cu): sides up to
+// kSmallMaxL in sw_sweep_noalloc (which then needs no scratch) and as the most
+// sw_batch_set_small takes; any L <= 256 would fit the CTA.
 constexpr int kSmallMaxL = 181;
-// sw_sweep takes the one-CTA path (any L <= 256 fits) up to kSmallSweepMaxL,
-// for calls of one sweep up to kSmallCallMaxL: a sweep costs the CTA less
-// than the tiled path's launches up to there, its first one twice that. Us
-// per sweep of a 100-sweep call (with one union-find over all runs, before
-// the segments): L = 64 9.0 (15.2), 100 14.5 (37.7), 144 20.7 (67.0); one
-// CTA / tiled: 160 24 / 30, 181 33 / 31, 256 57 / 30. One-sweep calls with
-// their read-back: L = 144 76 / 73, 160 80 / 73.
-constexpr int kSmallSweepMaxL = 160;
-constexpr int kSmallCallMaxL = 144;
-inline bool small_sweep(int L, int n) { return L <= kSmallCallMaxL || (L <= kSmallSweepMaxL && n > 1); }
+// sw_sweep takes this path up to the side where the tiled path (128 x 32
+// tiles) becomes as fast. A sweep costs the CTA less than the tiles' launches,
+// a call's first one and the E/M pass after its last one twice that, and the
+// assignment rule a block for every root instead of one for 128 sites. Us a
+// sweep of a call of n sweeps with its read-back, one CTA / tiles:
+//   flip      n = 1    96 30.9 / 35.2   104 36.3 / 37.2   112 37.7 / 37.2   144 46.5 / 37.2
+//             n = 2   128 27.9 / 29.0   132 31.7 / 31.3
+//             n = 4   144 26.6 / 26.8   148 28.1 / 27.8
+//             n = 20  156 23.8 / 24.8   160 24.4 / 23.4
+//             n = 100  64  8.6 / 20.9    96 12.4 / 21.6   156 22.7 / 24.3   160 23.2 / 22.9
+//   assign    n = 1    96 34.4 / 36.8   104 40.5 / 38.6
+//             n = 2   112 30.7 / 31.7   120 31.9 / 31.6
+//             n = 4   124 26.7 / 28.1   128 27.4 / 27.2
+//             n = 20  132 25.8 / 26.6   136 26.6 / 26.4   160 31.6 / 25.2
+//             n = 100 132 24.7 / 25.9   140 26.0 / 25.9
+inline int small_sweep_max_L(int n, bool assign) {
+  if (assign) return n == 1 ? 96 : n < 4 ? 112 : n < 16 ? 124 : 132;
+  return n == 1 ? 104 : n < 4 ? 128 : n < 16 ? 144 : 156;
+}
 struct SmallArgs {
   int L;
   uint32_t thr;    // C3
