@@ -98,9 +98,34 @@ SWEEP_MODEL_BYTES_PER_SITE = 10  # read spins, write+read int32 labels, write sp
 # as for Ising (the state bytes take the place of the spins); phase 3 reads
 # the 16-bit tile roots, border-root and root masks, slot count, the tile's
 # slot states and the halo's slots and slot states, and writes the states.
-MS = 2 * (TW + TH)
-POTTS_BYTES_PER_TILE = (PHASE_BYTES_PER_TILE[0] + PHASE_BYTES_PER_TILE[1]
-                        + 2 * TW * TH + 2 * 4 * RW + 4 + MS + 3 * (TH + TW) + TW * TH)
+def potts_bytes_per_tile(tw: int, th: int) -> int:
+    pb, ms, rw = phase_bytes_per_tile(tw, th), 2 * (tw + th), (tw // 32) * th
+    return pb[0] + pb[1] + 2 * tw * th + 2 * 4 * rw + 4 + ms + 3 * (th + tw) + tw * th
+
+
+def potts_tile(L: int) -> tuple[int, int]:
+    """Tile of the Potts path (as the library chooses it)."""
+    return (128, 32) if L <= 1024 else (128, 64)
+
+
+def chain_bytes_per_tile(tw: int, th: int, strip_h: int) -> int:
+    """Algorithmic bytes of a sweep inside a multi-sweep call without
+    statistics: the merge phases (which then write the next sweep's draws)
+    and the fused launch where the shape has it (phases 1 and 3 take the same
+    block), else the one-sweep phases."""
+    pb = phase_bytes_per_tile(tw, th)
+    return pb[1] + 8 * (tw // 32) * th + pb[4] if th == 32 * strip_h else pb[0] + pb[1] + pb[2]
+
+
+def phi4_bytes_per_site(sites: int) -> float:
+    """Algorithmic bytes per site of one phi^4 update inside a call: bricks
+    (binary32 projection 4 in; parent 4 and bond bits 1 out), unite and roots
+    (bond bits 1 in each; the parent walks are data dependent and not
+    counted), reflect (parent 4 in; projection 8 in and field 32 in and out
+    for the half of the sites that flip), E and M with the next update's
+    projections (field 32 in, projections 8 and 4 out). Below 2^20 sites the
+    projections are a pass of their own and read the field again."""
+    return (4 + 4 + 1) + 1 + 1 + (4 + 0.5 * (8 + 64)) + (32 + 12) + (32 if sites < 1 << 20 else 0)
 
 
 def peaks():
@@ -604,9 +629,7 @@ def measure_other_configs(sw, torch, stream, flush):
     pb = phase_bytes_per_tile(tw1, th1)
     tiles = (1024 // tw1) * (1024 // th1)
     by_hist = (pb[0] + pb[1] + pb[2]) * tiles
-    # without statistics: the fused launch where the shape has it, else the
-    # one-sweep phases
-    by_fused = ((pb[1] + 8 * (tw1 // 32) * th1 + pb[4]) if shape1024 in (4, 6) else (pb[0] + pb[1] + pb[2])) * tiles
+    by_fused = chain_bytes_per_tile(tw1, th1, info["strip_h"]) * tiles
     g_hist = by_hist / (ms / n / 1e3) / 1e9
     g_fused = by_fused / (ms_nh / n / 1e3) / 1e9
     out["L1024_betac_cold_hist"] = {"su_s": 1024 * 1024 * n / (ms / 1e3), "us_per_sweep": 1e3 * ms / n,
@@ -661,22 +684,16 @@ def measure_other_configs(sw, torch, stream, flush):
             pt.sweep(10)
             ms = timed_sweeps(torch, stream, lambda: pt.sweep(n), n)
             pt.observables(10, n)
-        ntiles = -(-Lq // TW) * -(-Lq // TH)
-        gbs = POTTS_BYTES_PER_TILE * ntiles / (ms / n / 1e3) / 1e9
+        twq, thq = potts_tile(Lq)
+        ntiles = -(-Lq // twq) * -(-Lq // thq)
+        gbs = potts_bytes_per_tile(twq, thq) * ntiles / (ms / n / 1e3) / 1e9
         out[f"potts_q3_L{Lq}_betac"] = {
             "su_s": Lq * Lq * n / (ms / 1e3), "us_per_sweep": 1e3 * ms / n, "sweeps": n,
-            "bytes_per_site": POTTS_BYTES_PER_TILE / (TW * TH), "achieved_gbs": gbs,
+            "bytes_per_site": potts_bytes_per_tile(twq, thq) / (twq * thq), "achieved_gbs": gbs,
             "frac_of_hbm": gbs / peak_gbs, "peak": f"{peak_gbs:.0f} GB/s ({peak_kind})"}
     # O(4) phi^4 multicluster updates at the paper's kappa = 0.304 (§5's
     # second table: L = 16..28, 10^4 updates), and L = 64 (16.8 M sites,
     # 0.5 GB of field) where the update's arrays no longer fit in L2.
-    # Algorithmic bytes per site of one update: project (field 32 in,
-    # projection 8 and parent 4 out), bonds (projection 8 in, bond bits 1
-    # out), unite (bond bits 1 in; the parent walks are data dependent and
-    # not counted), roots (parent 4 in and 4 out), reflect (parent 4, flip 1,
-    # projection 8 in; the field of the half of the sites that flip, 32 in
-    # and 32 out), observables (field 32 in).
-    phi4_bytes = (32 + 8 + 4) + (8 + 1) + 1 + (4 + 4) + (4 + 1 + 8 + 0.5 * 64) + 32
     out["phi4_kappa0.304"] = {}
     for Lp in (16, 28, 64):
         with sw.Phi4(Lp, 0.304, 6, stream=stream.cuda_stream) as f4:
@@ -684,13 +701,14 @@ def measure_other_configs(sw, torch, stream, flush):
             n4 = 200
             ms4 = timed_sweeps(torch, stream, lambda: f4.sweep(n4), n4)
             f4.observables(5, n4)
+        phi4_bytes = phi4_bytes_per_site(Lp**4)
         gbs = phi4_bytes * Lp**4 / (ms4 / n4 / 1e3) / 1e9
         out["phi4_kappa0.304"][f"L{Lp}"] = {"ms_per_update": ms4 / n4, "site_updates_s": Lp**4 * n4 / (ms4 / 1e3),
                                             "updates": n4, "minutes_per_1e4_updates": ms4 / n4 * 1e4 / 6e4,
                                             "bytes_per_site": phi4_bytes, "achieved_gbs": gbs,
                                             "frac_of_hbm": gbs / peak_gbs,
                                             "peak": f"{peak_gbs:.0f} GB/s ({peak_kind})",
-                                            "l2": "fits in L2" if 46 * Lp**4 < 100e6 else "exceeds L2"}
+                                            "l2": "fits in L2" if 49 * Lp**4 < 100e6 else "exceeds L2"}
     return out
 
 
