@@ -136,8 +136,9 @@ int sw_destroy(sw_lattice* h);
  * growth), SW_ECUDA. Device-side failures are reported by the next call that
  * synchronises. A small lattice (L up to 96 .. 156, by n and the rule) with
  * statistics off runs all n sweeps in one CTA-sized launch (the whole lattice
- * in shared memory) unless the environment variable SW_TILE_SHAPE was set at sw_create, which
- * keeps it on the tiled path; the results are the same. Between the sweeps
+ * in shared memory; under sw_timing one launch of phase 0) unless the
+ * environment variable SW_TILE_SHAPE was set at sw_create, which keeps it on
+ * the tiled path; the results are the same. Between the sweeps
  * of one call the bond draws of the next sweep (C5: they depend on the
  * seed, the counter and the site, not on the spins) are taken during the
  * current sweep's cross-tile merge; a later call whose first counter is the
@@ -350,9 +351,9 @@ int sw_batch_destroy(sw_batch* b);
  *  P5  Observables after each sweep, int64: E = -(number of edges joining
  *      equal states), M = number of sites in state 0.
  *  For q = 2 and beta = 2 beta_Ising this is the Ising sweep with the
- *  assignment rule (C6b), state 1 <-> spin -1. The sweep runs site-parallel
- *  kernels over global memory (a union-find over int32 parents). Rules of
- *  the Ising handle (ownership, streams, statuses) apply.
+ *  assignment rule (C6b), state 1 <-> spin -1. The sweep runs on the Ising
+ *  sweep's tiled path (128x32 tiles up to L = 1024, 128x64 above). Rules of
+ *  the Ising handle (ownership, streams, threads, statuses) apply.
  * --------------------------------------------------------------------------- */
 typedef struct sw_potts sw_potts;
 
@@ -413,8 +414,9 @@ int sw_potts_destroy(sw_potts* h);
  *      orthogonal to r).
  *  Observables per update, binary64: E = sum over the 4N edges of
  *  phi_x . phi_{x+mu}, M = sum_x phi_x (4 components). They are reduced in
- *  parallel, so they match a serial sum to rounding, not bit for bit; the
- *  field itself is bit-exact.
+ *  parallel (fields of 2^20 sites and more in 64-bit fixed point where its
+ *  grid holds the block's sites, else in binary64), so they match a serial sum
+ *  to rounding, not bit for bit; the field itself is bit-exact.
  * --------------------------------------------------------------------------- */
 typedef struct sw_phi4 sw_phi4;
 

@@ -80,8 +80,9 @@ int preferred_shape(int L) {
 // than one wave of 152 SMs; with 128 x 32 tiles twice as many CTAs share
 // each phase's latency, and in phase 3 a thread has one row word (one-row
 // strips) instead of two to walk. With these strips phases 1 and 3 take the
-// same block, so that chains run them in one launch: L = 256 44.5 -> 36.7
-// us a sweep, 1024 49.9 -> 40.3, with statistics 78 -> 64.
+// same block, so that chains run them in one launch: in calls of 20 sweeps
+// L = 256 took 44.5 us a sweep before and 36.7 with these tiles (24.9 since),
+// 1024 49.9 and 40.3, with statistics 78 and 64.
 int lattice_shape(int L) {
   const int p = preferred_shape(L);
   return p >= 0 ? p : L <= 1024 ? 7 : 6;

@@ -28,7 +28,7 @@
 
 namespace {
 
-constexpr int kNoallocShape = 6;  // 128 x 64 tiles, 2-row strips, as sw_sweep uses for L > 64
+constexpr int kNoallocShape = 6;  // 128 x 64 tiles, 2-row strips
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct ScratchLayout {

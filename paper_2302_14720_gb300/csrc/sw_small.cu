@@ -1,7 +1,8 @@
 // sw_small.cu -- whole sweeps of a small lattice in one CTA.
 //
-// A lattice of at most 256 x 256 sites fits one CTA's shared memory whole:
-// spins and bonds as bit masks, and a 16-bit label per site. One launch runs
+// A lattice of at most 256 x 256 sites would fit one CTA's shared memory whole
+// (spins and bonds as bit masks, and a 16-bit label per site); the launchers
+// take sides up to kSmallMaxL, past which the tiles are faster. One launch runs
 // n sweeps back to back with block barriers between the steps, so a small
 // lattice costs no cross-tile merge and no launch per phase. The steps and
 // their results are those of the tiled path:
