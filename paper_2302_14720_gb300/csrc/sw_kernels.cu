@@ -1641,7 +1641,11 @@ __device__ __forceinline__ bool phase3_body(P3Shared<WPR, TH, H, MODE>& S, uint3
           const int bin = log2_floor(sz);
           cnt += 1u;
           sq += sz * sz;
-          if (bin < 8) {
+          if (BF == 8) {
+            if (bin < 4) bins[0] += 1u << (8 * bin);
+            else if (bin < 8) bins[1] += 1u << (8 * (bin - 4));
+            else atomicAdd(&s_hist[2 + bin], 1ull);
+          } else if (bin < 8) {
 #pragma unroll
             for (int q = 0; q < 8 / PW; ++q)
               if (bin / PW == q) bins[q] += 1u << (BF * (bin % PW));
