@@ -33,6 +33,7 @@
 #include <stdlib.h>
 
 #include <cmath>
+#include <limits>
 #include <new>
 
 #include "sw.h"
@@ -268,7 +269,7 @@ constexpr int kSiteMask = 0x7fffffff;  // a parent entry without its decision bi
 
 template <int B0, int B1, int B2, int B3, int NT>
 __global__ void __launch_bounds__(NT)
-    phi4_brick_kernel(const double* a, const float* af, uint8_t* bonds, int* par, int L, double k4, uint32_t t,
+    phi4_brick_kernel(const double* a, const float* af, uint8_t* bonds, int* par, int L, double k4, float k4f, uint32_t t,
                       sw::KeySchedule ks, int* err) {
   sw::start_next();
   sw::after_previous();
@@ -281,9 +282,6 @@ __global__ void __launch_bounds__(NT)
   float* const s_af = reinterpret_cast<float*>(s_buf);  // [V] projections, then the warps' lists
   __shared__ int s_par[V];
   __shared__ uint8_t s_b[V];  // bits 0-3: bonds inside the brick, 4-7: bonds that leave it
-  // (k4 f) f stays in binary32's normal range, or vanishes, for |f| >= 2^-60
-  // unless k4 is below 2^-66: with NaN every edge takes the binary64 test
-  const float k4f = k4 == 0.0 || k4 >= 0x1p-66 ? __double2float_rn(k4) : __int_as_float(0x7fffffff);
   const uint32_t uL = (uint32_t)L, L2 = uL * uL, L3 = L2 * uL;
   uint32_t q = blockIdx.x;
   const uint32_t g0 = (uL + B0 - 1) / B0, g1 = (uL + B1 - 1) / B1, g2 = (uL + B2 - 1) / B2;
@@ -918,9 +916,15 @@ int direction(uint64_t seed, uint32_t t, Dir& d) {
 template <int B0, int B1, int B2, int B3, int NT>
 void launch_brick(sw_phi4* h) {
   const int L = h->L;
+  const double k4 = 4.0 * h->kappa;
+  // (k4 f) f stays in binary32's normal range, or vanishes, for |f| >= 2^-60
+  // unless k4 is below 2^-66: with NaN every edge takes the binary64 test.
+  // (Taken on the host: every thread's binary64 comparisons cost 2 us an update
+  // at L = 64.)
+  const float k4f = k4 == 0.0 || k4 >= 0x1p-66 ? (float)k4 : std::numeric_limits<float>::quiet_NaN();
   const unsigned g = (unsigned)((L + B0 - 1) / B0) * ((L + B1 - 1) / B1) * ((L + B2 - 1) / B2) * ((L + B3 - 1) / B3);
   sw::launch_after(phi4_brick_kernel<B0, B1, B2, B3, NT>, g, NT, 0, h->stream, h->a, h->af, h->bonds, h->par, L,
-                   4.0 * h->kappa, (uint32_t)h->t, h->ks, h->err);
+                   k4, k4f, (uint32_t)h->t, h->ks, h->err);
 }
 
 template <int UNITE_ROWS, int ROOT_ROWS>
