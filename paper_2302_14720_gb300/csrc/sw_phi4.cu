@@ -524,10 +524,8 @@ __global__ void phi4_reflect_kernel(F4* phi, const double* a, const int* par, in
 // E and M of the new field. GB300's binary64 rate is about 1/60 of its
 // integer rate, and E takes 24 binary64 operations a site: at L = 64 the
 // binary64 kernel below ran 739 us, all of it in that pipe; the fixed-point one
-// runs about 265 us (16.8M sites, 0.54 GB of field), bound by instruction
-// issue: 223 us on a grid of 54 bits that every block took unchecked, and 44 us
-// for the wider grid, the check and the ordered sum of the blocks (an update
-// 1010 -> 1054 us).
+// runs about 225 us (16.8M sites, 0.54 GB of field), bound by instruction
+// issue, its check of the field's range (below) included.
 // Large lattices therefore sum in 64-bit fixed point: with 2^T above every
 // |phi| (T from the largest component, which the projection kernel leaves in
 // *top; a reflection keeps the length of phi), a component c becomes the
@@ -549,36 +547,39 @@ struct Fix4 {
   int64_t v[4];
 };
 
-// d 2^(58-T) rounded to the nearest integer, ties to even; shift0 = T + 1027.
-// A double is m 2^(e - 1086) with m its mantissa from bit 63 down, so the
-// result is m >> (T + 1028 - e), taken with one more bit and a sticky bit.
-// (Components just below the exact range lose a bit or two, so exact ties are
-// common and a fixed direction for them would be a bias that grows with the
-// sites.) lost: a bit of d fell off the grid.
-__device__ __forceinline__ int64_t to_fixed(double d, int shift0, bool& lost) {
+// d 2^(58-T) rounded to the nearest integer, ties away from zero; shift0 = T +
+// 1027. A double is m 2^(e - 1086) with m its mantissa from bit 63 down, so the
+// result is m >> (T + 1028 - e), taken with one more bit. (Ties are common just
+// below the exact range, where a component loses a bit or two: about 1 % of
+// components, so that their fixed direction adds some 2^-62 a site to M. On a
+// grid of 54 bits half of the components had them, and M was 1e-14 off.)
+__device__ __forceinline__ int64_t to_fixed(double d, int shift0) {
   const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
   const uint64_t m = ((uint64_t)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
   const uint32_t sh = (uint32_t)(shift0 - (int)((hi >> 20) & 0x7ffu));
-  uint64_t x, back;
+  uint64_t x;
   asm("shr.b64 %0, %1, %2;" : "=l"(x) : "l"(m), "r"(sh));  // shifts past 63 give 0
-  asm("shl.b64 %0, %1, %2;" : "=l"(back) : "l"(x), "r"(sh));
-  const uint32_t up = back != m ? 1u : (uint32_t)(x >> 1) & 1u;
-  lost = (back != m || (x & 1u)) && ((hi << 1) | lo) != 0u;  // (a zero has no leading bit to lose)
   const int64_t s = (int32_t)hi >> 31;
-  return ((int64_t)((x + up) >> 1) ^ s) - s;
+  return ((int64_t)((x + 1u) >> 1) ^ s) - s;
 }
 __device__ __forceinline__ Fix4 to_fixed(const F4& f, int shift0) {
-  bool lost;
-  return Fix4{{to_fixed(f.x, shift0, lost), to_fixed(f.y, shift0, lost), to_fixed(f.z, shift0, lost),
-               to_fixed(f.w, shift0, lost)}};
+  return Fix4{{to_fixed(f.x, shift0), to_fixed(f.y, shift0), to_fixed(f.z, shift0), to_fixed(f.w, shift0)}};
 }
-// The same, with the components that lost bits counted in the bytes of `lost`.
-__device__ __forceinline__ Fix4 to_fixed(const F4& f, int shift0, uint32_t& lost) {
-  bool l0, l1, l2, l3;
-  const Fix4 r{{to_fixed(f.x, shift0, l0), to_fixed(f.y, shift0, l1), to_fixed(f.z, shift0, l2),
-                to_fixed(f.w, shift0, l3)}};
-  lost = (l0 ? 1u : 0u) | (l1 ? 1u << 8 : 0u) | (l2 ? 1u << 16 : 0u) | (l3 ? 1u << 24 : 0u);
-  return r;
+
+// Whether d 2^(58-T) is no integer: the T + 1028 - e lowest bits of m (all of
+// them from 64 on) are not all 0. A zero has no leading bit to lose.
+__device__ __forceinline__ bool off_grid(double d, int shift0) {
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  const uint64_t m = ((uint64_t)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
+  const int above = max(63 - shift0 + (int)((hi >> 20) & 0x7ffu), 0);
+  uint64_t below;
+  asm("shl.b64 %0, %1, %2;" : "=l"(below) : "l"(m), "r"(above));
+  return below != 0u && ((hi << 1) | lo) != 0u;
+}
+// The components of f off the grid, counted in the bytes.
+__device__ __forceinline__ uint32_t off_grid(const F4& f, int shift0) {
+  return (off_grid(f.x, shift0) ? 1u : 0u) | (off_grid(f.y, shift0) ? 1u << 8 : 0u) |
+         (off_grid(f.z, shift0) ? 1u << 16 : 0u) | (off_grid(f.w, shift0) ? 1u << 24 : 0u);
 }
 
 // The block's sums of v[0..4], in threads 0..4. The five values are reduced
@@ -690,7 +691,7 @@ constexpr int64_t kLargeSites = 1 << 20;
 //
 // PROJECT: the same pass takes the projections of the next update, which read
 // the same field and are bound by the binary64 pipe while the sums are bound
-// by integer issue: 303 us together, 222 + 156 apart (L = 64, the 54-bit grid).
+// by integer issue: 303 us together, 222 + 156 apart (L = 64).
 template <bool PROJECT>
 __global__ void __launch_bounds__(kObserveThreads)
     phi4_observe_fixed_kernel(const F4* phi, int L, int64_t n, const uint32_t* top, int steps, double* part,
@@ -738,12 +739,14 @@ __global__ void __launch_bounds__(kObserveThreads)
   uint32_t am[4] = {0u, 0u, 0u, 0u}, ae = 0u, own_lost, up_lost, nlost = 0u;  // high words of |.|; counts by byte
   const F4 first = phi[(size_t)z0 * V + sc];
   if (PROJECT && have) project(first, (size_t)z0 * V + sc);
-  Fix4 own = to_fixed(first, shift0, own_lost);
+  Fix4 own = to_fixed(first, shift0);
+  own_lost = off_grid(first, shift0);
   for (int z = z0; z < z1; ++z) {
     const F4* slice = phi + (size_t)z * V;
     const F4 fu = phi[(size_t)(z + 1 == L ? 0 : z + 1) * V + sc];
     if (PROJECT && have && z + 1 < z1) project(fu, (size_t)(z + 1) * V + sc);
-    const Fix4 up = to_fixed(fu, shift0, up_lost);
+    const Fix4 up = to_fixed(fu, shift0);
+    up_lost = off_grid(fu, shift0);
     const F4 g2 = slice[n2];
     longlong2(&buf)[2][kObserveThreads] = s_x[z & 1];
     buf[0][threadIdx.x] = make_longlong2(own.v[0], own.v[1]);
